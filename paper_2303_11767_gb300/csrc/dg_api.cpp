@@ -189,6 +189,7 @@ StageArgs<T> base_args(dg_ctx *h, const RowTab<T> *rows, double href)
     a.status = h->d_status;
     a.nlon = h->nlon;
     a.nlat = h->nlat;
+    a.nlat_mesh = h->nlat_g;
     a.halo_s = h->gs;
     a.halo_n = h->gn;
     a.href = (T)href;

@@ -37,9 +37,15 @@ template <typename T>
 __device__ __forceinline__ T rcp(T x);
 template <>
 __device__ __forceinline__ double rcp<double>(double x) { return 1.0 / x; }
-// FP32: the SFU reciprocal (<= 2 ulp), far inside the FP32 tolerance
+// FP32: the SFU reciprocal alone (<= 1 ulp; __fdividef(1, x) scales its
+// argument around it, for depths that do not occur)
 template <>
-__device__ __forceinline__ float rcp<float>(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ float rcp<float>(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
 template <typename T>
 __device__ __forceinline__ T wave_sqrt(T x);
@@ -47,7 +53,12 @@ template <>
 __device__ __forceinline__ double wave_sqrt<double>(double x) { return sqrt(x); }
 // FP32: x * rsqrt(x) on the SFU; only feeds the Rusanov dissipation speed
 template <>
-__device__ __forceinline__ float wave_sqrt<float>(float x) { return x * rsqrtf(x); }
+__device__ __forceinline__ float wave_sqrt<float>(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return x * y;
+}
 
 // Finiteness of many values with one test at the end: chk = fma(x, 0, chk)
 // for each x stays 0 while every x is finite and becomes NaN (for good) at

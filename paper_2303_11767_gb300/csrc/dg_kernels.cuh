@@ -882,9 +882,57 @@ constexpr size_t stage_smem_bytes()
     return SmemMap<T, N, W>::BYTES;
 }
 
+#ifdef DG_REAL_IS_F32
+}  // namespace dgk
+#include "dg_stage_ept.cuh"
+namespace dgk {
+// Tiles of 16 x 8 (degrees 3 and 4) and 32 x 4 elements: the wider one has the
+// larger ring but one row per warp (degree 2 720x360 29.7 against 31.4 us,
+// degree 4 1440x720 453 against 380).
+template <int N, int TX, int TY, int MINB>
+int launch_ept_n(const StageArgs<float> &a, cudaStream_t s)
+{
+    using GE = EptGeo<N, TX, TY>;
+    using K = void (*)(const StageArgs<float>);
+    const K k00 = ept_stage_kernel<N, TX, TY, MINB, 0, 0>, k01 = ept_stage_kernel<N, TX, TY, MINB, 0, 1>,
+            k10 = ept_stage_kernel<N, TX, TY, MINB, 1, 0>, k11 = ept_stage_kernel<N, TX, TY, MINB, 1, 1>;
+    static std::atomic<unsigned long long> attr_set{0};   // handles on other host threads may launch too
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    if (!(attr_set.load(std::memory_order_acquire) >> dev & 1ull)) {
+        for (K k : {k00, k01, k10, k11})
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GE::BYTES) != cudaSuccess)
+                return 1;
+        attr_set.fetch_or(1ull << dev, std::memory_order_release);   // setting it twice is harmless
+    }
+    dim3 grid((a.nlon + TX - 1) / TX, (a.nlat + TY - 1) / TY);
+    const K k = a.inc ? (a.out_base ? k11 : k10) : (a.out_base ? k01 : k00);
+    if (launch_pdl(k, grid, dim3(GE::NT), GE::BYTES, s, a) != cudaSuccess) return 1;
+    return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
+}
+#endif
+
 template <typename T, int N>
 int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
 {
+#ifdef DG_REAL_IS_F32
+    // One thread per element where the mesh has enough elements for it; else
+    // N lanes per element, whose tiles have the shorter chain (one tile takes
+    // 8 instead of 13 us at degree 4).  The line lies where both take the same
+    // time; us per stage, lanes / threads: degree 4 180x90 13.9 / 13.2, 360x180
+    // 40.5 / 34.8, 1440x720 586 / 380; degree 3 180x90 5.85 / 8.5, 360x180 16.5
+    // / 14.5, 1440x720 235 / 204; degree 2 120x60 5.1 / 6.1, 241x121 8.6 / 7.2,
+    // 720x360 53.9 / 29.7; degree 1 120x60 3.4 / 4.0, 720x360 18.7 / 14.7.
+    // It counts the whole mesh's rows, so that a latitude band of a mesh runs
+    // the kernel of the whole mesh and gets its bits.
+    if constexpr (N >= 2) {
+        constexpr long long least = N == 5 ? 14000 : N == 4 ? 40000 : 18000;
+        if ((long long)a.nlon * a.nlat_mesh >= least) {
+            if constexpr (N >= 4) return launch_ept_n<N, 16, 8, N == 5 ? 3 : 4>(a, s);
+            else return launch_ept_n<N, 32, 4, N == 3 ? 5 : 6>(a, s);
+        }
+    }
+#endif
     constexpr int W = DG_WARPS;
     using GE = Geo<N, W>;
     const size_t smem = stage_smem_bytes<T, N, W>();
@@ -947,6 +995,7 @@ __global__ void __launch_bounds__(32 * W, 24 / W) ensemble_kernel(const EnsArgs<
         A.status = E.status;
         A.nlon = m.nlon;
         A.nlat = m.nlat;
+        A.nlat_mesh = m.nlat;
         A.halo_s = A.halo_n = 0;
         A.href = m.href;
         A.P0 = m.P0;

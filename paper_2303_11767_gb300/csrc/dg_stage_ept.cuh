@@ -1,0 +1,630 @@
+// dg_stage_ept.cuh -- the fused FP32 stage with one thread per element, for
+// meshes with enough elements to fill the chip that way (the dispatch rule is
+// at launch_stage_n).  Included by dg_kernels.cuh.
+//
+// What bounds it and why this shape.  The stage with N lanes per element
+// (stage_tile) is bound by the load/store pipe: at degree 4 it spent 63
+// shared-memory and 41-104 global wavefronts per element on transposes
+// between the passes and on row accesses of 5 words, 68-74 % of the pipe's
+// peak, with the FMA pipe at 25-32 %.  Here an element's two-dimensional
+// contractions run in the registers of one thread, without transposes:
+//   * the tile's modes cross HBM / L2 in aligned 16-byte blocks (stage state
+//     base + increment added on the way into shared memory; the tendency
+//     goes back through shared memory and the Runge-Kutta update runs on the
+//     same flat 16-byte blocks);
+//   * every thread reads its element's modes from shared memory, where the
+//     element stride is odd in words (or in 16-byte units), so the lanes hit
+//     different banks, and overwrites them with the Gauss-point values;
+//   * the volume integral contracts over lambda first, with the constant
+//     basis tables as operands of the FMAs, one theta row of Gauss points at
+//     a time; the inverse mass matrix is folded into the theta contraction
+//     (per-row tables QT, PT), where the E / W edge fluxes join as two more
+//     columns of the same table;
+//   * only edge traces and edge fluxes are exchanged between threads.
+// The halo ring's traces are summed in the owning thread's order and the flux
+// routines are the shared ones, so both tiles of a tile boundary (or both
+// bands of a band boundary) get that edge's flux from the same bits.
+#pragma once
+
+namespace dgk {
+
+template <int N, int TX, int TY>
+struct EptGeo {
+    static constexpr int NP = N * N, EL = 3 * NP;
+    static constexpr int NT = TX * TY;                  // threads of the block, one per element
+    static constexpr int RPW = 32 / TX;                 // tile rows per warp
+    static constexpr bool VEC = NP % 4 == 0;            // a field is whole 16-byte blocks
+    // element stride in shared memory: an odd number of words, or of 16-byte
+    // blocks where the modes are read as float4
+    static constexpr int ES = VEC ? ((EL / 4) % 2 ? EL : EL + 4) : EL;
+    // one tile row of elements; where a row may start anywhere in a 16-byte
+    // block (EL odd) it lands at the same offset within one, and the second
+    // row of a warp continues the bank pattern of the first
+    static constexpr int ROW = VEC ? TX * ES : TX * EL + 32;
+    static constexpr int SLOT0 = VEC ? ES : (EL + 3 + 3) / 4 * 4;
+    static constexpr int SLOT = (SLOT0 / 4) % 2 ? SLOT0 : SLOT0 + 4;   // one W / E ring element
+    static constexpr int C1 = TX + 1, R1 = TY + 1;
+    static constexpr int M_OFF = 0;                              // modes, then Gauss values, then tendencies
+    static constexpr int TE_OFF = M_OFF + TY * ROW;              // E traces [f][k][row][1 + col], col -1: W ring
+    static constexpr int TN_OFF = TE_OFF + 3 * N * TY * C1;      // N traces [f][k][1 + row][col], row -1: S ring
+    static constexpr int RW_OFF = TN_OFF + 3 * N * R1 * TX;      // W traces of the E ring [f][k][row]
+    static constexpr int RS_OFF = RW_OFF + 3 * N * TY;           // S traces of the N ring [f][k][col]
+    // the ring's modes, dead once its traces are known; then the edge fluxes
+    static constexpr int U_OFF = (RS_OFF + 3 * N * TX + 3) / 4 * 4;
+    static constexpr int RING_LEN = 2 * ROW + 2 * TY * SLOT;
+    static constexpr int FW_OFF = U_OFF;                         // W-edge fluxes [f][k][row][col]
+    static constexpr int FS_OFF = FW_OFF + 3 * N * TY * C1;      // S-edge fluxes [f][k][row][col]
+    static constexpr int FLUX_LEN = 3 * N * (TY * C1 + R1 * TX);
+    static constexpr int LEN = U_OFF + (RING_LEN > FLUX_LEN ? RING_LEN : FLUX_LEN);
+    static constexpr size_t BYTES = sizeof(float) * (size_t)LEN;
+    static_assert(32 % TX == 0 && NT % 32 == 0, "a warp holds whole tile rows");
+    static_assert((TX * EL) % 4 == 0 && ROW % 4 == 0 && SLOT % 4 == 0, "16-byte blocks");
+};
+
+// position of a value within its 16-byte block
+__device__ __forceinline__ int ept_lead(const float *p)
+{
+    return (int)((reinterpret_cast<uintptr_t>(p) >> 2) & 3);
+}
+
+__device__ __forceinline__ float4 ept_ld4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+
+// A field value (h) or the pair (hu, hv), which share every basis
+// coefficient: one paired FMA does both momenta, each rounded as the scalar.
+__device__ __forceinline__ float ept_fma(float c, float x, float acc) { return fma(c, x, acc); }
+__device__ __forceinline__ float2 ept_fma(float c, float2 x, float2 acc) { return __ffma2_rn(bc2(c), x, acc); }
+__device__ __forceinline__ float ept_mul(float c, float x) { return c * x; }
+__device__ __forceinline__ float2 ept_mul(float c, float2 x) { return __fmul2_rn(bc2(c), x); }
+template <typename V>
+__device__ __forceinline__ V ept_zero();
+template <>
+__device__ __forceinline__ float ept_zero<float>() { return 0.f; }
+template <>
+__device__ __forceinline__ float2 ept_zero<float2>() { return bc2(0.f); }
+// value at p of field f0 (V = float), or of fields f0 and f0 + 1 (stride apart)
+template <typename V>
+__device__ __forceinline__ V ept_get(const float *p, int stride);
+template <>
+__device__ __forceinline__ float ept_get<float>(const float *p, int) { return *p; }
+template <>
+__device__ __forceinline__ float2 ept_get<float2>(const float *p, int stride) { return make_float2(p[0], p[stride]); }
+__device__ __forceinline__ void ept_put(float *p, int, float v) { *p = v; }
+__device__ __forceinline__ void ept_put(float *p, int stride, float2 v) { p[0] = v.x, p[stride] = v.y; }
+
+// N consecutive values at p (per field), 16 bytes at a time where N is 4
+template <typename V, int N>
+__device__ __forceinline__ void ept_get_row(const float *p, int stride, V *o)
+{
+    if constexpr (N == 4 && sizeof(V) == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(p);
+        o[0] = v.x, o[1] = v.y, o[2] = v.z, o[3] = v.w;
+    } else if constexpr (N == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(p), w = *reinterpret_cast<const float4 *>(p + stride);
+        o[0] = make_float2(v.x, w.x), o[1] = make_float2(v.y, w.y);
+        o[2] = make_float2(v.z, w.z), o[3] = make_float2(v.w, w.w);
+    } else {
+#pragma unroll
+        for (int a = 0; a < N; ++a) o[a] = ept_get<V>(p + a, stride);
+    }
+}
+template <typename V, int N>
+__device__ __forceinline__ void ept_put_row(float *p, int stride, const V *o)
+{
+    if constexpr (N == 4 && sizeof(V) == 4) {
+        *reinterpret_cast<float4 *>(p) = make_float4(o[0], o[1], o[2], o[3]);
+    } else if constexpr (N == 4) {
+        *reinterpret_cast<float4 *>(p) = make_float4(o[0].x, o[1].x, o[2].x, o[3].x);
+        *reinterpret_cast<float4 *>(p + stride) = make_float4(o[0].y, o[1].y, o[2].y, o[3].y);
+    } else {
+#pragma unroll
+        for (int a = 0; a < N; ++a) ept_put(p + a, stride, o[a]);
+    }
+}
+
+// Values at the Gauss points of one field (or the momentum pair) from its
+// modes at me, written over them, and its edge traces: S and W returned, N
+// and E written for the neighbours (point k at tn + k tn_k, te + k te_k,
+// fields tn_f, te_f apart).
+template <typename V, int N>
+__device__ __forceinline__ void ept_values(const BasisTab<float> &B, float *me, V *trS, V *trW, float *tn, int tn_k,
+                                           int tn_f, float *te, int te_k, int te_f)
+{
+    constexpr int NP = N * N;
+    V t1[N][N], se[N], sw[N];
+#pragma unroll
+    for (int b = 0; b < N; ++b) {
+        V row[N];
+        ept_get_row<V, N>(me + b * N, NP, row);
+        se[b] = sw[b] = ept_zero<V>();
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            se[b] = ept_fma(B.SE[a], row[a], se[b]);
+            sw[b] = ept_fma(B.SW[a], row[a], sw[b]);
+        }
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            t1[b][q] = ept_zero<V>();
+#pragma unroll
+            for (int a = 0; a < N; ++a) t1[b][q] = ept_fma(B.LV[a][q], row[a], t1[b][q]);
+        }
+    }
+#pragma unroll
+    for (int al = 0; al < N; ++al) {
+        V ts = ept_zero<V>(), tnv = ept_zero<V>();
+#pragma unroll
+        for (int b = 0; b < N; ++b) {
+            ts = ept_fma(B.SW[b], t1[b][al], ts);
+            tnv = ept_fma(B.SE[b], t1[b][al], tnv);
+        }
+        trS[al] = ts;
+        ept_put(tn + al * tn_k, tn_f, tnv);
+        V y[N];
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            y[q] = ept_zero<V>();
+#pragma unroll
+            for (int b = 0; b < N; ++b) y[q] = ept_fma(B.LV[b][q], t1[b][al], y[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < N; ++q) t1[q][al] = y[q];
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        V tw = ept_zero<V>(), tev = ept_zero<V>();
+#pragma unroll
+        for (int b = 0; b < N; ++b) {
+            tw = ept_fma(B.LV[b][k], sw[b], tw);
+            tev = ept_fma(B.LV[b][k], se[b], tev);
+        }
+        trW[k] = tw;
+        ept_put(te + k * te_k, te_f, tev);
+    }
+#pragma unroll
+    for (int be = 0; be < N; ++be) ept_put_row<V, N>(me + be * N, NP, t1[be]);
+}
+
+// N / S lift of one field (or pair): kk[b][a] = CSW[b] sum_al w L_a gs - CSE[b] sum_al w L_a gn
+template <typename V, int N>
+__device__ __forceinline__ void ept_lift(const BasisTab<float> &B, const RowTab<float> *RT, const float *fs, int k_stride,
+                                         int f_stride, int row_stride, V (*kk)[N])
+{
+    V zs[N], zn[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) zs[a] = zn[a] = ept_zero<V>();
+#pragma unroll
+    for (int al = 0; al < N; ++al) {
+        const V gs = ept_get<V>(fs + al * k_stride, f_stride), gn = ept_get<V>(fs + al * k_stride + row_stride, f_stride);
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            zs[a] = ept_fma(B.WLV[a][al], gs, zs[a]);
+            zn[a] = ept_fma(B.WLV[a][al], gn, zn[a]);
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < N; ++b) {
+        const float cs = __ldg(&RT->CSW[b]), cn = -__ldg(&RT->CSE[b]);
+#pragma unroll
+        for (int a = 0; a < N; ++a) kk[b][a] = ept_fma(cs, zs[a], ept_mul(cn, zn[a]));
+    }
+}
+
+__device__ __forceinline__ float4 ept_state4(const float *base, const float *inc, bool has_inc, long long o)
+{
+    float4 v = ept_ld4(base + o);
+    if (has_inc) {
+        const float4 d = ept_ld4(inc + o);
+        v.x += d.x, v.y += d.y, v.z += d.z, v.w += d.w;
+    }
+    return v;
+}
+
+template <int N, int TX, int TY, int INC, int FIN>
+__device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int by, float *sm)
+{
+    using GE = EptGeo<N, TX, TY>;
+    constexpr int NP = GE::NP, EL = GE::EL, ES = GE::ES, ROW = GE::ROW, NT = GE::NT, RPW = GE::RPW;
+    constexpr int C1 = GE::C1, R1 = GE::R1;
+    constexpr bool VEC = GE::VEC;
+    const BasisTab<float> &B = c_basis[N - 1];
+    const float *const incp = A.inc;
+    const bool has_inc = INC == 0 ? false : INC == 1 ? true : incp != nullptr;
+    const bool fin = FIN == 0 ? false : FIN == 1 ? true : A.out_base != nullptr;
+
+    float *const M = sm + GE::M_OFF;
+    float *const TE = sm + GE::TE_OFF, *const TN = sm + GE::TN_OFF;
+    float *const RW = sm + GE::RW_OFF, *const RS = sm + GE::RS_OFF;
+    float *const RING = sm + GE::U_OFF;
+    float *const FW = sm + GE::FW_OFF, *const FS = sm + GE::FS_OFF;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cx = lane % TX, ry = warp * RPW + lane / TX;
+    const int i0 = bx * TX, j0 = by * TY;
+    const int Gv = min(TX, A.nlon - i0), Wv = min(TY, A.nlat - j0);
+    const bool valid = cx < Gv && ry < Wv;
+    const int j = j0 + (ry < Wv ? ry : 0);
+    const float href = A.href, gg = A.g;
+    const float ga_l = A.galpha ? A.galpha[0] : 0.f, ga_t = A.galpha ? A.galpha[1] : 0.f;
+    const RowTab<float> *const RT = A.rows + j;
+    unsigned st = 0;
+    float hmin = INFINITY;   // smallest depth at the Gauss points
+
+    // ---- S0: the tile's stage state, flat 16-byte blocks, each warp its rows.
+    // Block c of a row holds the values 4 c - lead .. of its segment.
+    auto row_off = [&](int jj) -> long long { return ((long long)jj * A.nlon + i0) * EL; };
+    auto blk_at = [](int c) -> int { return VEC ? (c / (EL / 4)) * ES + (c % (EL / 4)) * 4 : 4 * c; };
+    constexpr int RB = (TX * EL + 3 + 3) / 4, RBL = (RB + 31) / 32;   // blocks of a row, per lane
+#pragma unroll
+    for (int rr = 0; rr < RPW; ++rr) {
+        const int r = warp * RPW + rr;
+        const long long o = row_off(j0 + r);
+        const int ld = VEC ? 0 : ept_lead(A.base + o);
+        const int nb = r < Wv ? (ld + Gv * EL + 3) / 4 : 0;
+        const float *const pb = A.base + (o - ld) + 4 * lane, *const pi = has_inc ? incp + (o - ld) + 4 * lane : nullptr;
+        float4 v[RBL], d[RBL];
+#pragma unroll
+        for (int t = 0; t < RBL; ++t) {
+            if (lane + 32 * t < nb) {
+                v[t] = ept_ld4(pb + 128 * t);
+                if (has_inc) d[t] = ept_ld4(pi + 128 * t);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < RBL; ++t) {
+            if (lane + 32 * t < nb) {
+                if (has_inc) v[t].x += d[t].x, v[t].y += d[t].y, v[t].z += d[t].z, v[t].w += d[t].w;
+                *reinterpret_cast<float4 *>(M + r * ROW + blk_at(lane + 32 * t)) = v[t];
+            }
+        }
+    }
+
+    // ---- S0 ring: the elements around the tile (S row, N row, W and E
+    //      columns; periodic in lambda, none across a pole)
+    const bool hasS = j0 > 0 || A.halo_s, hasN = j0 + Wv < A.nlat || A.halo_n;
+    const int iW = i0 > 0 ? i0 - 1 : A.nlon - 1, iE = i0 + Gv < A.nlon ? i0 + Gv : 0;
+    const long long oS = row_off(j0 - 1), oN = row_off(j0 + Wv);
+    const int ldS = VEC ? 0 : ept_lead(A.base + oS), ldN = VEC ? 0 : ept_lead(A.base + oN);
+    auto col_off = [&](int s) -> long long {   // W ring elements s < TY, then E
+        return ((long long)(j0 + (s < TY ? s : s - TY)) * A.nlon + (s < TY ? iW : iE)) * EL;
+    };
+    {
+        const int nS = hasS ? (ldS + Gv * EL + 3) / 4 : 0, nN = hasN ? (ldN + Gv * EL + 3) / 4 : 0;
+#pragma unroll 2
+        for (int c = tid; c < nS; c += NT)
+            *reinterpret_cast<float4 *>(RING + blk_at(c)) = ept_state4(A.base, incp, has_inc, oS - ldS + 4 * c);
+#pragma unroll 2
+        for (int c = tid; c < nN; c += NT)
+            *reinterpret_cast<float4 *>(RING + ROW + blk_at(c)) = ept_state4(A.base, incp, has_inc, oN - ldN + 4 * c);
+        constexpr int PPS = VEC ? EL / 4 : (EL + 3 + 3) / 4;   // blocks that may hold a value of one element
+#pragma unroll 2
+        for (int v = tid; v < 2 * TY * PPS; v += NT) {
+            const int s = v / PPS, c = v - s * PPS;
+            if ((s < TY ? s : s - TY) < Wv) {
+                const long long o = col_off(s);
+                const int ld = VEC ? 0 : ept_lead(A.base + o);
+                if (4 * c < ld + EL)
+                    *reinterpret_cast<float4 *>(RING + 2 * ROW + s * GE::SLOT + 4 * c) =
+                        ept_state4(A.base, incp, has_inc, o - ld + 4 * c);
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---- S1: Gauss-point values of the own element, S4: its traces.  The W
+    //      and S traces stay in registers, E and N go to the neighbours.
+    float *const me = M + ry * ROW + (VEC ? 0 : ept_lead(A.base + row_off(j))) + cx * ES;
+    float trW0[N], trS0[N];      // h
+    float2 trW1[N], trS1[N];     // (hu, hv)
+    {
+        float *const tn = TN + (ry + 1) * TX + cx, *const te = TE + ry * C1 + cx + 1;
+        constexpr int KN = R1 * TX, KE = TY * C1;
+        ept_values<float, N>(B, me, trS0, trW0, tn, KN, N * KN, te, KE, N * KE);
+        ept_values<float2, N>(B, me + NP, trS1, trW1, tn + N * KN, KN, N * KN, te + N * KE, KE, N * KE);
+    }
+
+    // ---- S4 ring: one item per (ring element, field), its traces on the side
+    //      facing the tile, in the order of the owning thread
+    {
+        const int nS = hasS ? Gv : 0, nN = hasN ? Gv : 0;
+        const int items = 3 * (nS + nN + 2 * Wv);
+#pragma unroll 1
+        for (int it = tid; it < items; it += NT) {
+            const int r = it / 3, f = it - 3 * r;
+            const float *src;
+            float *dst;
+            int stride;
+            float acc[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) acc[k] = 0.f;
+            if (r < nS + nN) {   // theta edge: sum_b L_b(+-1) (sum_a L_a(xi_k) u[b][a])
+                const bool north = r >= nS;
+                const int c = north ? r - nS : r;
+                src = RING + (north ? ROW + ldN : ldS) + c * ES + f * NP;
+                dst = north ? RS + f * N * TX + c : TN + f * N * R1 * TX + c;
+                stride = north ? TX : R1 * TX;
+#pragma unroll
+                for (int b = 0; b < N; ++b) {
+                    float row[N], s[N];
+#pragma unroll
+                    for (int a = 0; a < N; ++a) row[a] = src[b * N + a];
+                    colsum<float, N>(B.LV, row, s);
+                    const float cb = north ? B.SW[b] : B.SE[b];   // the north ring's S trace
+#pragma unroll
+                    for (int k = 0; k < N; ++k) acc[k] = fma(cb, s[k], acc[k]);
+                }
+            } else {             // lambda edge: sum_b L_b(eta_k) (sum_a L_a(+-1) u[b][a])
+                const int s0 = r - nS - nN;
+                const bool east = s0 >= Wv;
+                const int w = east ? s0 - Wv : s0, slot = east ? TY + w : w;
+                src = RING + 2 * ROW + slot * GE::SLOT + (VEC ? 0 : ept_lead(A.base + col_off(slot))) + f * NP;
+                dst = east ? RW + f * N * TY + w : TE + (f * N * TY + w) * C1;
+                stride = east ? TY : TY * C1;
+#pragma unroll
+                for (int b = 0; b < N; ++b) {
+                    float s = 0.f;
+#pragma unroll
+                    for (int a = 0; a < N; ++a) s = fma(east ? B.SW[a] : B.SE[a], src[b * N + a], s);
+#pragma unroll
+                    for (int k = 0; k < N; ++k) acc[k] = fma(B.LV[b][k], s, acc[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < N; ++k) dst[k * stride] = acc[k];
+        }
+    }
+    __syncthreads();
+
+    // ---- S5: Rusanov fluxes, each edge once: every element its W and S edge,
+    //      the tile's E column and N row as separate items
+    {
+        float L[3], o[3];
+        if (valid) {
+            const bool south = j > 0 || A.halo_s;
+            const float cgs = A.cG * __ldg(&RT->ce_s);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                float Rr[3];
+#pragma unroll
+                for (int f = 0; f < 3; ++f) {
+                    L[f] = TE[((f * N + k) * TY + ry) * C1 + cx];
+                }
+                Rr[0] = trW0[k], Rr[1] = trW1[k].x, Rr[2] = trW1[k].y;
+                rusanov_lam(L, Rr, href, gg, A.cF, o, st, ga_l);
+#pragma unroll
+                for (int f = 0; f < 3; ++f) FW[((f * N + k) * TY + ry) * C1 + cx] = o[f];
+                if (south) {
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) {
+                        L[f] = TN[((f * N + k) * R1 + ry) * TX + cx];
+                    }
+                    Rr[0] = trS0[k], Rr[1] = trS1[k].x, Rr[2] = trS1[k].y;
+                    rusanov_th(L, Rr, href, gg, cgs, o, st, ga_t);
+                } else {   // pole edge: zero flux
+                    o[0] = o[1] = o[2] = 0.f;
+                }
+#pragma unroll
+                for (int f = 0; f < 3; ++f) FS[((f * N + k) * R1 + ry) * TX + cx] = o[f];
+            }
+        }
+        unsigned sb = 0;
+        const int nE = Wv * N, nN = Gv * N;
+#pragma unroll 1
+        for (int it = tid; it < nE + nN; it += NT) {
+            float Rr[3];
+            if (it < nE) {
+                const int k = it / Wv, w = it - k * Wv;
+#pragma unroll
+                for (int f = 0; f < 3; ++f) {
+                    L[f] = TE[((f * N + k) * TY + w) * C1 + Gv];
+                    Rr[f] = RW[(f * N + k) * TY + w];
+                }
+                rusanov_lam(L, Rr, href, gg, A.cF, o, sb, ga_l);
+#pragma unroll
+                for (int f = 0; f < 3; ++f) FW[((f * N + k) * TY + w) * C1 + Gv] = o[f];
+            } else {
+                const int r = it - nE, k = r / Gv, c = r - k * Gv;
+                if (hasN) {
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) {
+                        L[f] = TN[((f * N + k) * R1 + Wv) * TX + c];
+                        Rr[f] = RS[(f * N + k) * TX + c];
+                    }
+                    rusanov_th(L, Rr, href, gg, A.cG * __ldg(&A.rows[j0 + Wv - 1].ce_n), o, sb, ga_t);
+                } else {   // pole edge: zero flux
+                    o[0] = o[1] = o[2] = 0.f;
+                }
+#pragma unroll
+                for (int f = 0; f < 3; ++f) FS[((f * N + k) * R1 + Wv) * TX + c] = o[f];
+            }
+        }
+        if (sb) atomicOr(A.status, sb);
+    }
+    __syncthreads();
+
+    // ---- S6 N/S lift (through C_j^-1 L(+-1)), S2 fluxes and sources, S3
+    //      volume integral and E/W lift, S7 inverse mass matrix
+    float k0[N][N];      // h, [b][a]
+    float2 k1[N][N];     // (hu, hv)
+    {
+        constexpr int KN = R1 * TX;
+        const float *const fs = FS + ry * TX + cx;
+        ept_lift<float, N>(B, RT, fs, KN, N * KN, TX, k0);
+        ept_lift<float2, N>(B, RT, fs + N * KN, KN, N * KN, TX, k1);
+    }
+#pragma unroll 1
+    for (int be = 0; be < N; ++be) {
+        float x0[N];
+        float2 x1[N];
+        ept_get_row<float, N>(me + be * N, NP, x0);
+        ept_get_row<float2, N>(me + NP + be * N, NP, x1);
+        const float c = __ldg(&RT->cosn[be]), s = __ldg(&RT->sinn[be]), cGc = A.cG * c;
+        float Y10[N], Y20[N];    // coefficients of QT and PT: h
+        float2 Y11[N], Y21[N];   // (hu, hv)
+        {
+            constexpr int KE = TY * C1;
+            const float *const fw = FW + be * KE + ry * C1 + cx;
+            const float w0 = fw[0], e0 = fw[1];
+            const float2 w1 = ept_get<float2>(fw + N * KE, N * KE), e1 = ept_get<float2>(fw + N * KE + 1, N * KE);
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                Y10[a] = ept_fma(B.SW[a], w0, ept_mul(-B.SE[a], e0));
+                Y11[a] = ept_fma(B.SW[a], w1, ept_mul(-B.SE[a], e1));
+                Y20[a] = 0.f;
+                Y21[a] = bc2(0.f);
+            }
+        }
+#pragma unroll
+        for (int al = 0; al < N; ++al) {
+            const float hp = x0[al], hu = x1[al].x, hv = x1[al].y;
+            const float h = href + hp;
+            hmin = fmin(hmin, h);
+            const float rh = rcp(h);
+            const float u = hu * rh, v = hv * rh;
+            const float P = hp * gg * fma(0.5f, hp, href);
+            const float F0 = A.cF * hu, G0 = cGc * hv;
+            const float2 F1 = __fmul2_rn(bc2(A.cF), f2(fma(hu, u, P), hu * v));
+            const float2 G1 = __fmul2_rn(bc2(cGc), f2(hv * u, fma(hv, v, P)));
+            const float K = s * fma(A.twoOmega, c, u * A.invR);
+            const float2 S1 = f2(K * hv, fma(-K, hu, -(P * s * A.invR)));
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                const float wd = B.WLD[a][al], wl = B.WLV[a][al];
+                if (a > 0) {   // L_0' = 0
+                    Y10[a] = ept_fma(wd, F0, Y10[a]);
+                    Y11[a] = ept_fma(wd, F1, Y11[a]);
+                }
+                Y11[a] = ept_fma(wl, S1, Y11[a]);
+                Y20[a] = ept_fma(wl, G0, Y20[a]);
+                Y21[a] = ept_fma(wl, G1, Y21[a]);
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < N; ++b) {
+            const float qt = __ldg(&RT->QT[be][b]), pt = __ldg(&RT->PT[be][b]);
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                k0[b][a] = ept_fma(pt, Y20[a], ept_fma(qt, Y10[a], k0[b][a]));
+                k1[b][a] = ept_fma(pt, Y21[a], ept_fma(qt, Y11[a], k1[b][a]));
+            }
+        }
+    }
+    // h <= 0 at a Gauss point; a NaN depth makes the tendency NaN (below)
+    if (!(hmin > 0.f)) st |= DG_STATUS_NONPHYSICAL;
+#pragma unroll
+    for (int b = 0; b < N; ++b) {
+        k1[b][0].y = fma(A.P0, __ldg(&RT->rho[b]), k1[b][0].y);
+        ept_put_row<float, N>(me + b * N, NP, k0[b]);
+        ept_put_row<float2, N>(me + NP + b * N, NP, k1[b]);
+    }
+    __syncwarp();
+
+    // ---- S8: combine and store, flat 16-byte blocks, each warp its rows,
+    //      EB blocks of a lane at a time (their loads in flight together)
+    {
+        const float cdt = A.cc * A.dt, adt = A.ca * A.dt;
+        float chk = 0.f;   // non-finite tendency or state: NaN (nf_acc)
+        // u^{n+1} = (base + lo) + delta with an error-free two-sum, so
+        // increments far below one ulp of the state survive
+        auto two_sum = [&](float2 delta, float2 bs, float2 lo, float2 &ob, float2 &ol) {
+            const float2 s1 = __fadd2_rn(bs, delta);
+            const float2 bp = __fadd2_rn(s1, neg2(bs));
+            const float2 err = __fadd2_rn(__fadd2_rn(bs, neg2(__fadd2_rn(s1, neg2(bp)))), __fadd2_rn(delta, neg2(bp)));
+            const float2 l1 = __fadd2_rn(lo, err);
+            ob = __fadd2_rn(s1, l1);
+            ol = __fadd2_rn(l1, neg2(__fadd2_rn(ob, neg2(s1))));
+        };
+        // two values of a block: the outputs asked for (pi: increment, pa: accumulator, pb / pl: new state)
+        auto combine = [&](float2 k, float2 iv, float2 av, float2 bv, float2 lv, float2 &pi, float2 &pa, float2 &pb, float2 &pl) {
+            chk = nf_acc(k.x, nf_acc(k.y, chk));
+            const float2 ci = __fmul2_rn(bc2(A.ci), iv);
+            pi = __ffma2_rn(bc2(cdt), k, ci);
+            pa = __ffma2_rn(bc2(adt), k, av);
+            if (fin) {
+                two_sum(__ffma2_rn(bc2(cdt), k, __ffma2_rn(bc2(A.cd), av, ci)), bv, lv, pb, pl);
+                chk = nf_acc(pb.x, nf_acc(pb.y, chk));
+            }
+        };
+        constexpr int EB = FIN == 0 ? RBL : (RBL + 1) / 2;
+#pragma unroll 1
+        for (int rr = 0; rr < RPW; ++rr) {
+            const int r = warp * RPW + rr;
+            if (r >= Wv) break;
+            const long long o = row_off(j0 + r);
+            const int ld = VEC ? 0 : ept_lead(A.base + o), end = ld + Gv * EL, nb = (end + 3) / 4;
+#pragma unroll 1
+            for (int c0 = lane; c0 < nb; c0 += 32 * EB) {
+                const long long at0 = o - ld + 4 * c0;
+                float4 i4[EB], a4[EB], b4[EB], l4[EB];
+#pragma unroll
+                for (int t = 0; t < EB; ++t) {
+                    const long long at = at0 + 128 * t;
+                    i4[t] = a4[t] = b4[t] = l4[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (c0 + 32 * t < nb) {
+                        if (has_inc) i4[t] = ept_ld4(incp + at);
+                        if (A.acc_in) a4[t] = ept_ld4(A.acc_in + at);
+                        if (fin) b4[t] = ept_ld4(A.base + at);
+                        if (fin && A.lo) l4[t] = ept_ld4(A.lo + at);
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < EB; ++t) {
+                    const int c = c0 + 32 * t;
+                    if (c >= nb) break;
+                    const long long at = at0 + 128 * t;
+                    float4 kv = *reinterpret_cast<const float4 *>(M + r * ROW + blk_at(c));
+                    if (A.src) {
+                        const float4 s4 = ept_ld4(A.src + at);
+                        kv.x += s4.x, kv.y += s4.y, kv.z += s4.z, kv.w += s4.w;
+                    }
+                    if (VEC || (4 * c >= ld && 4 * c + 4 <= end)) {
+                        float2 pi[2], pa[2], pb[2], pl[2];
+                        combine(f2(kv.x, kv.y), f2(i4[t].x, i4[t].y), f2(a4[t].x, a4[t].y), f2(b4[t].x, b4[t].y),
+                                f2(l4[t].x, l4[t].y), pi[0], pa[0], pb[0], pl[0]);
+                        combine(f2(kv.z, kv.w), f2(i4[t].z, i4[t].w), f2(a4[t].z, a4[t].w), f2(b4[t].z, b4[t].w),
+                                f2(l4[t].z, l4[t].w), pi[1], pa[1], pb[1], pl[1]);
+                        auto put = [&](float *p, const float2 *v) {
+                            *reinterpret_cast<float4 *>(p + at) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+                        };
+                        if (A.out_rhs) *reinterpret_cast<float4 *>(A.out_rhs + at) = kv;
+                        if (A.inc_out) put(A.inc_out, pi);
+                        if (A.acc_out) put(A.acc_out, pa);
+                        if (fin) {
+                            put(A.out_base, pb);
+                            if (A.out_lo) put(A.out_lo, pl);
+                        }
+                    } else {   // a block shared with another tile's elements: its own values one by one
+                        const float k[4] = {kv.x, kv.y, kv.z, kv.w}, iv[4] = {i4[t].x, i4[t].y, i4[t].z, i4[t].w};
+                        const float av[4] = {a4[t].x, a4[t].y, a4[t].z, a4[t].w};
+                        const float bv[4] = {b4[t].x, b4[t].y, b4[t].z, b4[t].w};
+                        const float lv[4] = {l4[t].x, l4[t].y, l4[t].z, l4[t].w};
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            if (4 * c + m < ld || 4 * c + m >= end) continue;
+                            float2 pi, pa, pb, pl;
+                            combine(bc2(k[m]), bc2(iv[m]), bc2(av[m]), bc2(bv[m]), bc2(lv[m]), pi, pa, pb, pl);
+                            if (A.out_rhs) A.out_rhs[at + m] = k[m];
+                            if (A.inc_out) A.inc_out[at + m] = pi.x;
+                            if (A.acc_out) A.acc_out[at + m] = pa.x;
+                            if (fin) {
+                                A.out_base[at + m] = pb.x;
+                                if (A.out_lo) A.out_lo[at + m] = pl.x;
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        if (!isfinite(chk)) atomicOr(A.status, DG_STATUS_NONFINITE);   // of every lane: the blocks are not its own element's
+    }
+    if (st && valid) atomicOr(A.status, st);
+}
+
+template <int N, int TX, int TY, int MINB, int INC, int FIN>
+__global__ void __launch_bounds__(TX *TY, MINB) ept_stage_kernel(const StageArgs<float> A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_wait();
+    ept_tile<N, TX, TY, INC, FIN>(A, blockIdx.x, blockIdx.y, reinterpret_cast<float *>(smem_raw));
+    pdl_launch_dependents();   // at the end: triggered at the start, 240x120 at degree 4 took 18.9 instead of 15.0 us
+}
+
+}  // namespace dgk
