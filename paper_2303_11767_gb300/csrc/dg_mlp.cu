@@ -215,6 +215,12 @@ __global__ void to_bf16_kernel(const float *__restrict__ w, __nv_bfloat16 *__res
         wb[t] = __float2bfloat16_rn(w[t]);
 }
 
+}  // namespace
+
+#include "dg_mlp_fused.cuh"
+
+namespace {
+
 unsigned grid_for(size_t n) { return (unsigned)std::min<size_t>((n + 255) / 256, 4096); }
 
 }  // namespace
@@ -225,6 +231,11 @@ struct dg_mlp_ctx {
     size_t oW1, ob1, oW2, ob2, oW3, ob3;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *wb = nullptr;
+    // layers that fit the fused kernels: their 16-bit weights in the order of
+    // use; part and lpart hold the blocks' partial gradients and errors, and
+    // the layer buffers below stay empty
+    bool fused = false;
+    __nv_bfloat16 *wt = nullptr;
     float *norm = nullptr;    // in_mean[nin], in_std[nin], out_mean[nout], out_std[nout]
     float *rownorm = nullptr; // optional per latitude row: out_mean[nlat][nout], out_std[nlat][nout]
     int rownorm_nlat = 0;
@@ -243,6 +254,7 @@ void free_mlp(dg_mlp_ctx *c)
                      c->part})
         cudaFree(p);
     cudaFree(c->wb);
+    cudaFree(c->wt);
     cudaFree(c->lpart);
     delete c;
 }
@@ -309,9 +321,41 @@ void backward(dg_mlp_ctx *c, const float *x, int batch, cudaStream_t s)
     bias_grad_kernel<<<(c->H + 127) / 128, 128, 0, s>>>(c->dA, batch, c->H, g + c->ob1);
 }
 
-dg_status loss_and_grad(dg_mlp_ctx *c, const float *x, const float *t, int batch, double *loss)
+// 16-bit copies of the parameters
+void refresh_weights(dg_mlp_ctx *c, cudaStream_t s)
+{
+    to_bf16_kernel<<<grid_for(c->np), 256, 0, s>>>(c->w, c->wb, c->np);
+    if (c->fused) fused_weights_kernel<<<grid_for(c->np), 256, 0, s>>>(c->w, c->wt, c->nin, c->nout, c->np);
+}
+
+struct AdamStep {
+    float lr, b1, b2, eps, c1, c2;
+};
+
+// Loss and gradient of a batch; with `adam` also the optimiser step, its
+// moments corrected for step number c->step + 1.
+dg_status loss_and_grad(dg_mlp_ctx *c, const float *x, const float *t, int batch, double *loss, const AdamStep *adam)
 {
     cudaStream_t s = c->stream;
+    if (c->fused) {
+        const int blocks = (batch + FS - 1) / FS;
+        fused_mlp_kernel<true><<<blocks, 256, F_BYTES, s>>>(x, t, batch, c->nin, c->nout, c->wt, c->w, c->norm, nullptr, c->part,
+                                                             c->np, c->lpart);
+        const unsigned rb = (unsigned)((c->np + 63) / 64);
+        double *const lsum = c->lpart + FMAXB;
+        if (adam)
+            fused_reduce_kernel<true><<<rb, 256, 0, s>>>(c->part, c->lpart, blocks, c->np, c->nin, c->nout, c->g, lsum, c->w, c->m, c->v,
+                                                         c->wb, c->wt, adam->lr, adam->b1, adam->b2, adam->eps, adam->c1, adam->c2);
+        else
+            fused_reduce_kernel<false><<<rb, 256, 0, s>>>(c->part, c->lpart, blocks, c->np, c->nin, c->nout, c->g, lsum, c->w, c->m,
+                                                          c->v, c->wb, c->wt, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
+        double l = 0.0;
+        MCUDA(cudaMemcpyAsync(&l, lsum, sizeof l, cudaMemcpyDeviceToHost, s));
+        MCUDA(cudaStreamSynchronize(s));
+        *loss = l / ((double)batch * c->nout);
+        MCUDA(cudaPeekAtLastError());
+        return DG_OK;
+    }
     forward(c, x, batch, s);
     const int nb = 64;
     mse_kernel<<<nb, 256, 0, s>>>(c->Y, t, c->norm + 2 * c->nin, c->norm + 2 * c->nin + c->nout, batch, c->nout, c->dY,
@@ -323,6 +367,9 @@ dg_status loss_and_grad(dg_mlp_ctx *c, const float *x, const float *t, int batch
     double l = 0.0;
     for (double p : part) l += p;
     *loss = l / ((double)batch * c->nout);
+    if (adam)
+        adam_kernel<<<grid_for(c->np), 256, 0, s>>>(c->w, c->g, c->m, c->v, c->wb, c->np, adam->lr, adam->b1, adam->b2, adam->eps,
+                                                    adam->c1, adam->c2);
     MCUDA(cudaPeekAtLastError());
     return DG_OK;
 }
@@ -356,8 +403,14 @@ dg_status dg_mlp_create(int n_in, int n_hidden, int n_out, unsigned long long se
               cudaMalloc(&c->m, sizeof(float) * c->np) == cudaSuccess &&
               cudaMalloc(&c->v, sizeof(float) * c->np) == cudaSuccess &&
               cudaMalloc(&c->wb, sizeof(__nv_bfloat16) * c->np) == cudaSuccess &&
-              cudaMalloc(&c->norm, sizeof(float) * 2 * (n_in + n_out)) == cudaSuccess &&
-              cudaMalloc(&c->Z1, sizeof(float) * MAXB * n_hidden) == cudaSuccess &&
+              cudaMalloc(&c->norm, sizeof(float) * 2 * (n_in + n_out)) == cudaSuccess;
+    c->fused = n_hidden == FH && n_in <= FIN && n_out <= FOUT;
+    if (ok && c->fused)
+        ok = cudaMalloc(&c->wt, sizeof(__nv_bfloat16) * T_LEN) == cudaSuccess &&
+             cudaMalloc(&c->part, sizeof(float) * FMAXB * c->np) == cudaSuccess &&
+             cudaMalloc(&c->lpart, sizeof(double) * (FMAXB + 1)) == cudaSuccess;
+    else if (ok)
+        ok = cudaMalloc(&c->Z1, sizeof(float) * MAXB * n_hidden) == cudaSuccess &&
               cudaMalloc(&c->A1, sizeof(float) * MAXB * n_hidden) == cudaSuccess &&
               cudaMalloc(&c->Z2, sizeof(float) * MAXB * n_hidden) == cudaSuccess &&
               cudaMalloc(&c->A2, sizeof(float) * MAXB * n_hidden) == cudaSuccess &&
@@ -393,14 +446,19 @@ dg_status dg_mlp_create(int n_in, int n_hidden, int n_out, unsigned long long se
     for (int i = 0; i < n_in; ++i) norm[n_in + i] = 1.0f;
     for (int i = 0; i < n_out; ++i) norm[2 * n_in + n_out + i] = 1.0f;
     c->stream = nullptr;
-    if (cudaMemcpy(c->w, w.data(), sizeof(float) * c->np, cudaMemcpyHostToDevice) != cudaSuccess ||
+    if ((c->fused && (cudaMemset(c->wt, 0, sizeof(__nv_bfloat16) * T_LEN) != cudaSuccess ||   // (zero padding)
+                      cudaFuncSetAttribute(fused_mlp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_BYTES) !=
+                          cudaSuccess ||
+                      cudaFuncSetAttribute(fused_mlp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_BYTES) !=
+                          cudaSuccess)) ||
+        cudaMemcpy(c->w, w.data(), sizeof(float) * c->np, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->norm, norm.data(), sizeof(float) * norm.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->m, 0, sizeof(float) * c->np) != cudaSuccess ||
         cudaMemset(c->v, 0, sizeof(float) * c->np) != cudaSuccess) {
         free_mlp(c);
         return mfail(DG_ECUDA, "initial copy failed");
     }
-    to_bf16_kernel<<<grid_for(c->np), 256>>>(c->w, c->wb, c->np);
+    refresh_weights(c, c->stream);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         free_mlp(c);
         return mfail(DG_ECUDA, "initialisation failed");
@@ -430,7 +488,7 @@ dg_status dg_mlp_set_params(dg_mlp m, const float *params, size_t n)
 {
     if (!m || !params || n != m->np) return mfail(DG_EINVAL, "need %zu parameters", m ? m->np : 0);
     MCUDA(cudaMemcpy(m->w, params, sizeof(float) * n, cudaMemcpyHostToDevice));
-    to_bf16_kernel<<<grid_for(m->np), 256>>>(m->w, m->wb, m->np);
+    refresh_weights(m, m->stream);
     MCUDA(cudaDeviceSynchronize());
     return DG_OK;
 }
@@ -479,6 +537,13 @@ dg_status dg_mlp_set_row_normalization(dg_mlp m, int nlat, const float *out_mean
 dg_status dg_mlp_forward(dg_mlp m, const float *d_x, int batch, float *d_y)
 {
     if (!m || !d_x || !d_y || batch < 1 || batch > MAXB) return mfail(DG_EINVAL, "batch must be 1..%d", MAXB);
+    if (m->fused) {
+        fused_mlp_kernel<false><<<(batch + FS - 1) / FS, 256, F_BYTES, m->stream>>>(d_x, nullptr, batch, m->nin, m->nout, m->wt, m->w,
+                                                                                    m->norm, d_y, nullptr, m->np, nullptr);
+        MCUDA(cudaPeekAtLastError());
+        MCUDA(cudaStreamSynchronize(m->stream));
+        return DG_OK;
+    }
     forward(m, d_x, batch, m->stream);
     MCUDA(cudaMemcpyAsync(d_y, m->Y, sizeof(float) * batch * m->nout, cudaMemcpyDeviceToDevice, m->stream));
     MCUDA(cudaStreamSynchronize(m->stream));
@@ -491,7 +556,7 @@ dg_status dg_mlp_gradients(dg_mlp m, const float *d_x, const float *d_t, int bat
     if (!m || !d_x || !d_t || !grads || n != m->np || batch < 1 || batch > MAXB)
         return mfail(DG_EINVAL, "bad arguments (batch 1..%d, %zu gradients)", MAXB, m ? m->np : 0);
     double l = 0;
-    if (dg_status s = loss_and_grad(m, d_x, d_t, batch, &l)) return s;
+    if (dg_status s = loss_and_grad(m, d_x, d_t, batch, &l, nullptr)) return s;
     MCUDA(cudaMemcpy(grads, m->g, sizeof(float) * n, cudaMemcpyDeviceToHost));
     if (loss) *loss = l;
     return DG_OK;
@@ -502,13 +567,10 @@ dg_status dg_mlp_train_step(dg_mlp m, const float *d_x, const float *d_t, int ba
     if (!m || !d_x || !d_t || batch < 1 || batch > MAXB || !(lr > 0))
         return mfail(DG_EINVAL, "bad arguments (batch 1..%d, lr > 0)", MAXB);
     double l = 0;
-    if (dg_status s = loss_and_grad(m, d_x, d_t, batch, &l)) return s;
+    const float b1 = 0.9f, b2 = 0.999f, step = (float)(m->step + 1);
+    const AdamStep adam{(float)lr, b1, b2, 1e-8f, 1.0f - std::pow(b1, step), 1.0f - std::pow(b2, step)};
+    if (dg_status s = loss_and_grad(m, d_x, d_t, batch, &l, &adam)) return s;
     m->step++;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - std::pow(b1, (float)m->step), c2 = 1.0f - std::pow(b2, (float)m->step);
-    adam_kernel<<<grid_for(m->np), 256, 0, m->stream>>>(m->w, m->g, m->m, m->v, m->wb, m->np, (float)lr, b1, b2,
-                                                       1e-8f, c1, c2);
-    MCUDA(cudaPeekAtLastError());
     if (loss) *loss = l;
     return DG_OK;
 }
