@@ -197,6 +197,14 @@ StageArgs<T> base_args(dg_ctx *h, const RowTab<T> *rows, double href)
     // vector rho; the well-balanced option drops it (that state is steady)
     a.P0 = h->wb ? T(0) : (T)(0.5 * h->g * href * href);
     a.g = (T)h->g;
+    if (h->physics == 2) {   // the f-plane: no curvature, constant Coriolis parameter, periodic in y
+        a.nlat_mesh = h->nlat;
+        a.halo_s = a.halo_n = a.wrap = 1;
+        a.cF = (T)(2.0 * h->nlon / h->plen);
+        a.cG = (T)(2.0 * h->nlat / h->plen);
+        a.twoOmega = (T)h->fcor;
+        return a;
+    }
     a.cF = (T)(2.0 / (h->R * h->tab.dlam));
     a.cG = (T)(2.0 / (h->R * h->tab.dth));
     a.invR = (T)(1.0 / h->R);
@@ -256,9 +264,6 @@ int launch_plane(dg_ctx *h, const StageArgs<double> &a)
     pa.nx = h->nlon;
     pa.ny = h->nlat;
     pa.alpha_speed = h->alpha_speed;
-    pa.swe = h->physics == 2;
-    pa.g = h->g;
-    pa.fcor = h->fcor;
     return dg_launch_stage_plane(h->n, pa, h->stream);
 }
 
@@ -327,7 +332,7 @@ dg_status launch_stage_t(dg_ctx *h, double dt, int cur, const RowTab<T> *rows, i
             r = h->tc() ? dg_launch_stage_tc(h->n, h->prec - DG_PREC_FP32_TC_BF16, a, h->stream)
                         : dg_launch_stage<T>(h->n, a, h->stream);
         } else {
-            r = h->physics != 0 ? launch_plane(h, a) : dg_launch_stage<T>(h->n, a, h->stream);
+            r = h->physics == 1 ? launch_plane(h, a) : dg_launch_stage<T>(h->n, a, h->stream);
         }
         if (r) return fail(DG_ECUDA, "stage kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
         h->launches++;
@@ -619,12 +624,17 @@ dg_status dg_create_plane_swe(int nx, int ny, int degree, double L, double g, do
     h->plen = L;
     h->g = g;
     h->fcor = f;
-    if ((st = alloc_state_buffers(h)) != DG_OK) {
+    h->tab.rows = static_cast<RowTab<double> *>(std::calloc(ny, sizeof(RowTab<double>)));
+    if (!h->tab.rows) st = fail(DG_ENOMEM, "host allocation failed");
+    for (int j = 0; !st && j < ny; ++j) dg_plane_row(h->n, h->pbasis, h->tab.rows[j]);
+    if (!st) st = upload_basis_once(h->device);
+    if (!st) st = upload_rows<double>(h, &h->rows64);
+    if (!st) st = alloc_state_buffers(h);
+    if (st) {
         dg_destroy(h);
         *out = nullptr;
-        return st;
     }
-    return DG_OK;
+    return st;
 }
 
 dg_status dg_create_plane_advection(int nx, int ny, int degree, double bx, double by, int alpha_speed,
@@ -910,12 +920,10 @@ dg_status dg_rhs(dg_handle h, const double *modal_in, double *tend_out, size_t l
     void *in = h->I[0], *outb = h->I[1];
     if (h->physics != 0) {
         CUDA_TRY(cudaMemcpyAsync(in, modal_in, len * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-        StageArgs<double> a;
-        std::memset(&a, 0, sizeof a);
-        a.status = h->d_status;
+        StageArgs<double> a = base_args<double>(h, h->rows64, 0.0);
         a.base = static_cast<double *>(in);
         a.out_rhs = static_cast<double *>(outb);
-        if (launch_plane(h, a))
+        if (h->physics == 1 ? launch_plane(h, a) : dg_launch_stage<double>(h->n, a, h->stream))
             return fail(DG_ECUDA, "planar stage launch failed: %s", cudaGetErrorString(cudaGetLastError()));
         h->launches++;
         CUDA_TRY(cudaMemcpyAsync(tend_out, outb, len * sizeof(double), cudaMemcpyDeviceToHost, h->stream));

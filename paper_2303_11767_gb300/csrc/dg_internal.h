@@ -59,6 +59,9 @@ void dg_gauss_legendre(int n, double *x, double *w);
 double dg_legendre(int k, double x);
 double dg_legendre_deriv(int k, double x);
 int dg_build_tables(HostTables &t, int nlon, int nlat, int p, double R, double g);
+// The row table of the planar shallow-water problem of n = p + 1: a row of
+// the same element operator with cos = sin = 1 and the unit mass matrix.
+void dg_plane_row(int n, const BasisTab<double> &basis, RowTab<double> &r);
 void dg_free_tables(HostTables &t);
 
 // Stage-kernel launch description.  The time integration is written in
@@ -92,6 +95,7 @@ struct StageArgs {
     // of row nlat - 1 (halo_n) is a neighbour band's row, held in the state
     // arrays just before / after the band's own rows, instead of a pole
     int halo_s, halo_n;
+    int wrap;        // 1: periodic in the second direction too (the planar problem; halo_s = halo_n = 1)
     T href;          // reference depth: h = href + stored h
     T P0;            // g href^2 / 2 (pressure carried by the rho table)
     T g, cF, cG, invR, twoOmega;
@@ -199,8 +203,7 @@ int dg_mlp_launch_source(const dg_mlp_ctx *m, const float *base, const float *in
                          const double *c0, float *src, void *stream);
 bool dg_mlp_shape_is(const dg_mlp_ctx *m, int nin, int h, int nout);
 
-// dg_plane.cu: planar linear advection (one scalar, periodic unit square)
-// and planar shallow water on the f-plane (h, hu, hv; periodic square).
+// dg_plane.cu: planar linear advection (one scalar, periodic unit square).
 // k = M^{-1} h(u) with the FP64 stage semantics of StageArgs (href, rows, lo
 // unused); cx = 2 / dx, cy = 2 / dy; alpha_speed 1: Rusanov alpha = |beta|,
 // 0: |beta . n|.
@@ -209,8 +212,6 @@ struct PlaneArgs {
     BasisTab<double> basis;
     double bx, by, cx, cy;
     int nx, ny, alpha_speed;
-    int swe;          // 1: shallow water on the f-plane (3 fields) instead of advection
-    double g, fcor;   // gravity and the constant Coriolis parameter (swe)
 };
 int dg_launch_stage_plane(int n, const PlaneArgs &p, void *stream);
 

@@ -82,9 +82,8 @@ struct Geo {
     // touch distinct banks
     static constexpr int TRC = bank_free_stride(12 * N, N, 32 / N);   // traces W,E,S,N x 3 x N
     static constexpr int EFC = bank_free_stride(6 * N, N, 32 / N);    // edge fluxes W,S x 3 x N
-    static constexpr int HALO_MAX = 2 * W * N + 2 * G * N;
-    static_assert(HALO_MAX <= 32 * W, "halo items exceed the block");
-    static_assert(W * N + G * N <= 32 * W, "boundary flux items exceed the block");
+    static constexpr int HALO_MAX = 2 * W * N + 2 * G * N;   // halo trace points of a tile
+    static constexpr int EDGE_MAX = W * N + G * N;           // points of its E and N edges
 };
 
 // Shared-memory map of one tile, in elements of T: the warp buffers, the
@@ -323,8 +322,13 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
     const int nSe = hasS ? Gv : 0, nNe = hasN ? Gv : 0;
     const int nH = 2 * Wv + nSe + nNe;
     const int iW = i0 > 0 ? i0 - 1 : A.nlon - 1, iE = i0 + Gv < A.nlon ? i0 + Gv : 0;   // i0 + Gv <= nlon
-    // value offset of ring element h: W column, E column, S row, N row (hj =
-    // -1 is a neighbour band's row held just before row 0)
+    // the row south (north = false) or north of the tile: a neighbour band's
+    // rows -1 and nlat are held around the own rows, a periodic mesh wraps
+    auto ring_row = [&](bool north) -> int {
+        if (north) return A.wrap && j0 + Wv == A.nlat ? 0 : j0 + Wv;
+        return A.wrap && j0 == 0 ? A.nlat - 1 : j0 - 1;
+    };
+    // value offset of ring element h: W column, E column, S row, N row
     auto ring_off = [&](int h) -> long long {
         int hj, hi;
         if (h < 2 * Wv) {
@@ -334,7 +338,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
         } else {
             const int r = h - 2 * Wv;
             const bool north = r >= nSe;
-            hj = north ? j0 + Wv : j0 - 1;
+            hj = ring_row(north);
             hi = i0 + (north ? r - nSe : r);
         }
         return ((long long)hj * A.nlon + hi) * EL;
@@ -357,7 +361,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
             } else {
                 const int r = h - 2 * Wv;
                 const bool north = r >= nSe;
-                hj = north ? j0 + Wv : j0 - 1;
+                hj = ring_row(north);
                 hi = i0 + (north ? r - nSe : r);
             }
             const long long o = ((long long)hj * A.nlon + hi) * EL + c;
@@ -464,7 +468,56 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
     // ---- S4 halo: traces of the ring of neighbour elements facing the tile
     cp_async_wait_all();   // the ring's modes are in shared memory
     __syncthreads();
-    if constexpr (N >= 5) {
+    if constexpr (sizeof(T) == 8) {
+        // FP64: one item per (ring element, field) of a lambda edge, whose N
+        // traces share the row sums (2 N^2 multiply-adds on the pipe that bounds
+        // it), and per trace point of a theta edge, the same sums in the same
+        // order as the owning tile's
+        const int nWE = 3 * 2 * Wv, nSN = 3 * N * (nSe + nNe);
+        for (int it = tid; it < nWE + nSN; it += 32 * W) {
+            const T *hb, *hbi;
+            if (it < nWE) {
+                const int r = it / 3, f = it - 3 * r;
+                const bool east = r >= Wv;      // the east halo's W trace, the west halo's E trace
+                const int w = east ? r - Wv : r;
+                ring_at(r, hb, hbi);
+                hb += f * NP;
+                hbi += f * NP;
+                T acc[N];
+#pragma unroll
+                for (int kk = 0; kk < N; ++kk) acc[kk] = T(0);
+#pragma unroll
+                for (int b = 0; b < N; ++b) {
+                    T s = T(0);
+#pragma unroll
+                    for (int a = 0; a < N; ++a)
+                        s = fma(east ? B.SW[a] : B.SE[a], has_inc ? hb[b * N + a] + hbi[b * N + a] : hb[b * N + a], s);
+#pragma unroll
+                    for (int kk = 0; kk < N; ++kk) acc[kk] = fma(B.LV[b][kk], s, acc[kk]);
+                }
+                T *slot = trc + ((w + 1) * TW + (east ? Gv + 1 : 0)) * TRC + ((east ? 0 : 1) * 3 + f) * N;
+#pragma unroll
+                for (int kk = 0; kk < N; ++kk) slot[kk] = acc[kk];
+            } else {
+                const int q = it - nWE, r = q / (3 * N), fk = q - r * (3 * N), f = fk / N, kk = fk - f * N;
+                const bool north = r >= nSe;    // the north halo's S trace, the south halo's N trace
+                const int c = north ? r - nSe : r;
+                ring_at(2 * Wv + r, hb, hbi);
+                hb += f * NP;
+                hbi += f * NP;
+                T acc = T(0);
+#pragma unroll
+                for (int b = 0; b < N; ++b) {
+                    T s = T(0);
+#pragma unroll
+                    for (int a = 0; a < N; ++a)
+                        s = fma(B.LV[a][kk], has_inc ? hb[b * N + a] + hbi[b * N + a] : hb[b * N + a], s);
+                    acc = fma(north ? B.SW[b] : B.SE[b], s, acc);
+                }
+                trc[((north ? Wv + 1 : 0) * TW + c + 1) * TRC + ((north ? 2 : 3) * 3 + f) * N + kk] = acc;
+            }
+        }
+    } else if constexpr (N >= 5) {
         // degree 4: one item per (ring element, field), its N traces on the
         // side that faces the tile, each mode row read once (a third of the
         // instructions of one item per trace point; measured +9 % at 1440x720
@@ -535,8 +588,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
         // the same sums in the same order
         const int nWE = Wv * N;
         const int nS = hasS ? Gv * N : 0, nN = hasN ? Gv * N : 0;
-        const int it = tid;   // whole warps take halo items (no divergence inside a warp)
-        if (it < 2 * nWE + nS + nN) {
+        // whole warps take halo items (no divergence inside a warp), one each
+        // unless the tile is too short for its ring
+        auto halo_point = [&](int it) {
             int side, kk, sl, hh;
             if (it < 2 * nWE) {                 // west / east halo columns
                 const bool east = it >= nWE;
@@ -595,6 +649,11 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
                 }
                 slot[(side * 3 + f) * N + kk] = acc;
             }
+        };
+        if constexpr (GE::HALO_MAX <= 32 * W) {
+            if (tid < 2 * nWE + nS + nN) halo_point(tid);
+        } else {
+            for (int it = tid; it < 2 * nWE + nS + nN; it += 32 * W) halo_point(it);
         }
     }
     __syncthreads();
@@ -624,8 +683,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
             for (int f = 0; f < 3; ++f) ef[(own * 2 + 1) * 3 * N + f * N + k] = fx[f];
         }
         const int nE = Wv * N, nN = hasN ? Gv * N : 0;
-        const int it = 32 * W - 1 - tid;   // the last warps, which have no halo items
-        if (it < nE + nN) {
+        // the last warps, which have no halo items
+        for (int it = 32 * W - 1 - tid; it < nE + nN; it += 32 * W) {
             T L[3], R[3];
             if (it < nE) {                      // E edge of the last valid column
                 const int w = it / N, kk = it - (it / N) * N;
@@ -650,6 +709,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
 #pragma unroll
                 for (int f = 0; f < 3; ++f) ef[(su * 2 + 1) * 3 * N + f * N + kk] = fx[f];
             }
+            if constexpr (GE::EDGE_MAX <= 32 * W) break;
         }
     }
     __syncthreads();
@@ -912,37 +972,21 @@ int launch_ept_n(const StageArgs<float> &a, cudaStream_t s)
 }
 #endif
 
-template <typename T, int N>
-int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
+constexpr int DG_SMS = 152;   // SMs of a GB300
+
+template <typename T, int N, int W>
+int launch_stage_w(const StageArgs<T> &a, cudaStream_t s)
 {
-#ifdef DG_REAL_IS_F32
-    // One thread per element where the mesh has enough elements for it; else
-    // N lanes per element, whose tiles have the shorter chain (one tile takes
-    // 8 instead of 13 us at degree 4).  The line lies where both take the same
-    // time; us per stage, lanes / threads: degree 4 180x90 13.9 / 13.2, 360x180
-    // 40.5 / 34.8, 1440x720 586 / 380; degree 3 180x90 5.85 / 8.5, 360x180 16.5
-    // / 14.5, 1440x720 235 / 204; degree 2 120x60 5.1 / 6.1, 241x121 8.6 / 7.2,
-    // 720x360 53.9 / 29.7; degree 1 120x60 3.4 / 4.0, 720x360 18.7 / 14.7.
-    // It counts the whole mesh's rows, so that a latitude band of a mesh runs
-    // the kernel of the whole mesh and gets its bits.
-    if constexpr (N >= 2) {
-        constexpr long long least = N == 5 ? 14000 : N == 4 ? 40000 : 18000;
-        if ((long long)a.nlon * a.nlat_mesh >= least) {
-            if constexpr (N >= 4) return launch_ept_n<N, 16, 8, N == 5 ? 3 : 4>(a, s);
-            else return launch_ept_n<N, 32, 4, N == 3 ? 5 : 6>(a, s);
-        }
-    }
-#endif
-    constexpr int W = DG_WARPS;
     using GE = Geo<N, W>;
     const size_t smem = stage_smem_bytes<T, N, W>();
     // One kernel per stage kind (increment present or not, final stage or
     // not) up to p = 3, where the specialised kernels measured faster
     // (180x90: 6.28 -> 5.98 us per stage); one kernel reading the kind from
-    // its arguments at p = 4, where they did not (360x180: 43.2 -> 44.2 us).
+    // its arguments at p = 4, where they did not (360x180: 43.2 -> 44.2 us),
+    // and in FP64's short tiles (1 % there).
     using K = void (*)(const StageArgs<T>);
     K k00, k01, k10, k11;
-    if constexpr (N <= 4) {
+    if constexpr (N <= 4 && (sizeof(T) == 4 || W == DG_WARPS)) {
         k00 = stage_kernel<T, N, W, 0, 0>;
         k01 = stage_kernel<T, N, W, 0, 1>;
         k10 = stage_kernel<T, N, W, 1, 0>;
@@ -964,6 +1008,54 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     const K k = a.inc ? (a.out_base ? k11 : k10) : (a.out_base ? k01 : k00);
     if (launch_pdl(k, grid, dim3(32 * W), smem, s, a) != cudaSuccess) return 1;
     return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
+}
+
+template <typename T, int N>
+int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
+{
+#ifdef DG_REAL_IS_F32
+    // One thread per element where the mesh has enough elements for it; else
+    // N lanes per element, whose tiles have the shorter chain (one tile takes
+    // 8 instead of 13 us at degree 4).  The line lies where both take the same
+    // time; us per stage, lanes / threads: degree 4 180x90 13.9 / 13.2, 360x180
+    // 40.5 / 34.8, 1440x720 586 / 380; degree 3 180x90 5.85 / 8.5, 360x180 16.5
+    // / 14.5, 1440x720 235 / 204; degree 2 120x60 5.1 / 6.1, 241x121 8.6 / 7.2,
+    // 720x360 53.9 / 29.7; degree 1 120x60 3.4 / 4.0, 720x360 18.7 / 14.7.
+    // It counts the whole mesh's rows, so that a latitude band of a mesh runs
+    // the kernel of the whole mesh and gets its bits.
+    if constexpr (N >= 2) {
+        constexpr long long least = N == 5 ? 14000 : N == 4 ? 40000 : 18000;
+        if ((long long)a.nlon * a.nlat_mesh >= least) {
+            if constexpr (N >= 4) return launch_ept_n<N, 16, 8, N == 5 ? 3 : 4>(a, s);
+            else return launch_ept_n<N, 32, 4, N == 3 ? 5 : 6>(a, s);
+        }
+    }
+#endif
+    // Tile rows.  FP64 is bound by the FP64 pipe of the busiest SM: tiles per SM
+    // x rows x the cost of a row in a tile of that height (a short tile has more
+    // ring traces and evaluates more of its boundary edges twice).  Measured at
+    // 8, 4, 2, 1 rows (us per stage): 20x10 degree 1 36.4 23.8 23.3 26.8 (4 tiles
+    // of 8 rows ran on 4 SMs); 50x50 degree 3 69 44 44 48; 120x60 degree 2 52.6
+    // 53.3 46.2 50.3; 180x90 degree 3 138 143 154 180; 360x180 degree 4 906 821
+    // 901 1118: a row costs 1, 1.02, 1.2 and 1.5, and one-row tiles never win.
+    // FP32 takes 8 rows (90x45 degree 3 4.5 4.7 5.2 5.9; 180x90 5.9 6.2 7.6 11.9).
+    int w = DG_WARPS;
+    if (sizeof(T) == 8) {
+        double best = 0;
+        for (int c = DG_WARPS; c >= 2; c /= 2) {
+            const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((a.nlat + c - 1) / c);
+            const double work = (double)((tiles + DG_SMS - 1) / DG_SMS) * c * (c == 8 ? 1.0 : c == 4 ? 1.02 : 1.2);
+            if (c == DG_WARPS || work < best) {
+                best = work;
+                w = c;
+            }
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (w == 2) return launch_stage_w<T, N, 2>(a, s);
+        if (w == 4) return launch_stage_w<T, N, 4>(a, s);
+    }
+    return launch_stage_w<T, N, DG_WARPS>(a, s);
 }
 
 // ---------------------------------------------------------------- ensemble --
@@ -996,7 +1088,7 @@ __global__ void __launch_bounds__(32 * W, 24 / W) ensemble_kernel(const EnsArgs<
         A.nlon = m.nlon;
         A.nlat = m.nlat;
         A.nlat_mesh = m.nlat;
-        A.halo_s = A.halo_n = 0;
+        A.halo_s = A.halo_n = A.wrap = 0;
         A.href = m.href;
         A.P0 = m.P0;
         A.g = E.g;

@@ -203,3 +203,19 @@ int dg_build_tables(HostTables &t, int nlon, int nlat, int p, double R, double g
     }
     return 0;
 }
+
+void dg_plane_row(int n, const BasisTab<double> &basis, RowTab<double> &r)
+{
+    std::memset(&r, 0, sizeof r);
+    r.ce_s = r.ce_n = 1.0;
+    for (int b = 0; b < n; ++b) {
+        r.cosn[b] = r.sinn[b] = 1.0;
+        r.CSE[b] = basis.SE[b];
+        r.CSW[b] = basis.SW[b];
+        r.Ci[b][b] = 1.0;
+        for (int q = 0; q < n; ++q) {
+            r.Q[b][q] = r.QT[q][b] = basis.WLV[b][q];
+            r.PT[q][b] = basis.WLD[b][q];
+        }
+    }
+}
