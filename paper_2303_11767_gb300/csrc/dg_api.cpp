@@ -103,6 +103,7 @@ struct dg_ctx {
     long long aux_launches = 0;   // conversion, mass and wave-speed kernels
     dg_mlp_ctx *mlp = nullptr;    // learned source term (degree 1, FP32)
     float *src = nullptr;         // its per-stage modal output
+    double *src_part = nullptr;   // and partial sums of the mass in it
     std::vector<GraphEntry> graphs;
     double bx = 0, by = 0;       // planar advection velocity
     double plen = 1.0, fcor = 0; // planar domain side and f-plane Coriolis parameter
@@ -288,6 +289,22 @@ dg_status enqueue_global_speeds(dg_ctx *h, StageArgs<T> &a)
     return DG_OK;
 }
 
+// The attached network's source for the stage input a.base + a.inc.
+dg_status enqueue_source(dg_ctx *h, StageArgs<float> &a)
+{
+    const int r = dg_mlp_launch_source(h->mlp, a.base, a.inc, a.href, h->nlon, h->nlat, h->c0, h->src, h->src_part, h->stream);
+    if (r == 2) return fail(DG_EINVAL, "the network's row statistics belong to another mesh");
+    if (r) return fail(DG_ECUDA, "learned source launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    a.src = h->src;
+    a.src_part = h->src_part;
+    a.src_parts = dg_mlp_source_blocks((int)h->nel);
+    double area = 0.0;   // sum over the elements of the mass weight of mode 0
+    for (int j = 0; j < h->nlat; ++j) area += h->tab.C[(size_t)j * h->nphi];
+    a.src_area = area * h->nlon;
+    h->aux_launches += 1;
+    return DG_OK;
+}
+
 // Stage s of one RK step from u^n in base buffer `cur`.
 template <typename T>
 dg_status launch_stage_t(dg_ctx *h, double dt, int cur, const RowTab<T> *rows, int s)
@@ -315,16 +332,8 @@ dg_status launch_stage_t(dg_ctx *h, double dt, int cur, const RowTab<T> *rows, i
         a.cd = (T)pl[s].cd;
         a.dt = (T)dt;
         if constexpr (sizeof(T) == sizeof(float)) {
-            if (h->mlp) {
-                const int ms = dg_mlp_launch_source(h->mlp, reinterpret_cast<const float *>(a.base),
-                                                    reinterpret_cast<const float *>(a.inc), (float)h->href, h->nlon,
-                                                    h->nlat, h->c0, h->src, h->stream);
-                if (ms == 2) return fail(DG_EINVAL, "the network's row statistics belong to another mesh");
-                if (ms)
-                    return fail(DG_ECUDA, "learned source launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-                a.src = reinterpret_cast<const T *>(h->src);
-                h->aux_launches += 2;
-            }
+            if (h->mlp)
+                if (dg_status ms = enqueue_source(h, a)) return ms;
         }
         if (dg_status gs = enqueue_global_speeds<T>(h, a)) return gs;
         int r;
@@ -714,6 +723,7 @@ dg_status dg_destroy(dg_handle h)
     cudaFree(h->d_maxbits);
     cudaFree(h->galpha);
     cudaFree(h->src);
+    cudaFree(h->src_part);
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
     dg_free_tables(h->tab);
     delete h;
@@ -959,13 +969,8 @@ dg_status dg_rhs(dg_handle h, const double *modal_in, double *tend_out, size_t l
         StageArgs<float> a = base_args<float>(h, h->rows32, href);
         a.base = static_cast<float *>(in);
         a.out_rhs = static_cast<float *>(outb);
-        if (h->mlp) {   // the attached learned source is part of the tendency
-            const int ms = dg_mlp_launch_source(h->mlp, a.base, nullptr, (float)href, h->nlon, h->nlat, h->c0, h->src,
-                                                h->stream);
-            if (ms == 2) return fail(DG_EINVAL, "the network's row statistics belong to another mesh");
-            if (ms) return fail(DG_ECUDA, "learned source launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-            a.src = h->src;
-        }
+        if (h->mlp)   // the attached learned source is part of the tendency
+            if (dg_status ms = enqueue_source(h, a)) return ms;
         if (dg_status gs = enqueue_global_speeds<float>(h, a)) return gs;
         r = dg_launch_stage<float>(h->n, a, h->stream);
     }
@@ -1282,7 +1287,8 @@ dg_status dg_attach_mlp(dg_handle h, dg_mlp m)
     if (h->physics != 0 || h->p != 1 || h->prec != DG_PREC_FP32)
         return fail(DG_EUNSUPPORTED, "the learned source needs a degree-1 FP32 sphere solver");
     if (!dg_mlp_shape_is(m, 60, 128, 12)) return fail(DG_EINVAL, "the learned source needs a 60-128-128-12 network");
-    if (!h->src && cudaMalloc(&h->src, sizeof(float) * h->len) != cudaSuccess)
+    if ((!h->src && cudaMalloc(&h->src, sizeof(float) * h->len) != cudaSuccess) ||
+        (!h->src_part && cudaMalloc(&h->src_part, sizeof(double) * dg_mlp_source_blocks((int)h->nel)) != cudaSuccess))
         return fail(DG_ENOMEM, "cudaMalloc of the source buffer failed");
     h->mlp = m;
     return DG_OK;

@@ -85,7 +85,11 @@ struct StageArgs {
     T *acc_out;
     T *out_base;
     T *out_lo;
-    const T *src;    // optional modal source added to k (learned correction)
+    const T *src;    // optional modal source added to k (learned correction), after
+                     // (sum of src_part[0 .. src_parts)) / src_area is taken from mode 0 of h
+    const double *src_part;
+    int src_parts;
+    double src_area;
     const T *galpha; // global Rusanov mode: [max |u| + c, max |v| + c] of the stage input; null = local
     const RowTab<T> *rows;
     unsigned int *status;
@@ -199,8 +203,11 @@ int dg_launch_restrict(const double *fine, int fnlon, int fn, double *coarse, in
 
 // dg_mlp.cu: the learned source term of a degree-1 solver
 struct dg_mlp_ctx;
+// src: the modal source; part: dg_mlp_source_blocks(nel) partial sums of the
+// mass it would add (StageArgs::src_part).
 int dg_mlp_launch_source(const dg_mlp_ctx *m, const float *base, const float *inc, float href, int nlon, int nlat,
-                         const double *c0, float *src, void *stream);
+                         const double *c0, float *src, double *part, void *stream);
+int dg_mlp_source_blocks(int nel);
 bool dg_mlp_shape_is(const dg_mlp_ctx *m, int nin, int h, int nout);
 
 // dg_plane.cu: planar linear advection (one scalar, periodic unit square).

@@ -260,6 +260,18 @@ __device__ __forceinline__ void load_stage_row(const T *__restrict__ base, const
     }
 }
 
+// What is taken from mode 0 of h of the learned source so that it adds no
+// mass: the blocks' sums over the area, in a fixed order (every warp forms it
+// for itself).
+template <typename T>
+__device__ __forceinline__ T source_shift(const StageArgs<T> &A)
+{
+    double m = 0.0;
+    for (int v = threadIdx.x & 31; v < A.src_parts; v += 32) m += A.src_part[v];
+    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+    return (T)(m / A.src_area);
+}
+
 // One tile of G x W elements (tile column bx, tile row by) of one mesh.  The
 // modes of the tile's halo ring reach shared memory through asynchronous
 // contiguous copies issued at the start of the tile, so that their latency
@@ -832,11 +844,13 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
             }
         }
         kk[2][0] = fma(A.P0, rhok, kk[2][0]);
+        const T shift = N == 2 && A.src ? source_shift(A) : T(0);
         if (A.src && valid) {   // learned modal source, same layout as the state
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
                 T sv[N];
                 load_row<T, N>(A.src + e * EL + f * NP + k * N, sv);
+                if (f == 0 && k == 0) sv[0] -= shift;
 #pragma unroll
                 for (int a = 0; a < N; ++a) kk[f][a] += sv[a];
             }
@@ -1083,6 +1097,9 @@ __global__ void __launch_bounds__(32 * W, 24 / W) ensemble_kernel(const EnsArgs<
         A.out_lo = E.out_lo ? E.out_lo + m.off : nullptr;
         A.rows = E.rows + m.rows;
         A.src = nullptr;
+        A.src_part = nullptr;
+        A.src_parts = 0;
+        A.src_area = 0;
         A.galpha = nullptr;
         A.status = E.status;
         A.nlon = m.nlon;

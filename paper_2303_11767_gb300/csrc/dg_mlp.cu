@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -18,6 +19,7 @@
 #include <new>
 #include <vector>
 
+#include "dg_flux.cuh"
 #include "dg_internal.h"
 #include "../../include/dgswe.h"
 
@@ -581,138 +583,147 @@ dg_status dg_mlp_train_step(dg_mlp m, const float *d_x, const float *d_t, int ba
 
 namespace {
 
-// One CTA of 128 threads (one per hidden unit) evaluates the network for
-// SRC_EPC consecutive coarse elements of a degree-1 mesh: gather each
-// element's and its four neighbours' modes (zeros across a pole), normalise
-// them into shared memory, then every thread forms its hidden unit of the
-// first and of the second layer for all the CTA's elements (BF16 weights,
-// FP32 accumulation), and the outputs (element, q) are spread over the
-// threads.  Every sum starts at its bias and runs over inputs / units in
-// index order, exactly as an evaluation of one element at a time.  The
-// state is u_stage = base + inc with h stored relative to href (mode 0 of h
-// carries 2 href).
-constexpr int SRC_EPC = 8;
-
-__global__ void __launch_bounds__(128) mlp_source_kernel(
-    const float *__restrict__ base, const float *__restrict__ inc, float href, int nlon, int nlat,
-    const __nv_bfloat16 *__restrict__ wb, const float *__restrict__ wf, size_t ob1, size_t oW2, size_t ob2,
-    size_t oW3, size_t ob3, const float *__restrict__ norm, const float *__restrict__ rownorm,
-    float *__restrict__ src)
+// Block of 8 S threads: the network for S consecutive elements of a degree-1
+// mesh.  It gathers each element's and its four neighbours' modes (zeros
+// across a pole), normalises them into shared memory and runs the layers as
+// the training kernel does (4 elements x 4 units of a layer per thread, k-major
+// weights).  The state is u_stage = base + inc with h stored relative to href
+// (mode 0 of h carries 2 href).  The mass that the source would add,
+// sum_b w_j[b] s(h, a = 0, b) with w_j[b] the mass weights C_j[0][b] of the
+// element's row, is summed over the block into part: the stage kernel removes
+// the total from mode (0, 0) of h, spread over the area.
+//
+// The weights (51 KB) are read once per block before the wait for the previous
+// stage, so S is the smallest size that gives every SM at most one block.  At
+// 72x36, per stage: one thread per hidden unit reading its own weight row 46 us
+// and a single-block mass sum 13 us; now 15 us together.
+template <int S>
+__global__ void __launch_bounds__(8 * S) mlp_source_kernel(const float *__restrict__ base, const float *__restrict__ inc, float href,
+                                                           int nlon, int nlat, const __nv_bfloat16 *__restrict__ wt,
+                                                           const float *__restrict__ wf, const float *__restrict__ norm,
+                                                           const float *__restrict__ rownorm, const double *__restrict__ c0,
+                                                           float *__restrict__ src, double *__restrict__ part)
 {
-    constexpr int NIN = 60, H = 128, NOUT = 12, PER = 12, EPC = SRC_EPC;
-    static_assert(EPC * NOUT <= H, "one output per thread");
-    __shared__ float xs[EPC][NIN];
-    __shared__ float hs[EPC][H];
-    const int nel = nlon * nlat;
-    const int e0 = blockIdx.x * EPC;
-    const int t = threadIdx.x;
-    for (int v = t; v < EPC * NIN; v += H) {
-        const int el = v / NIN, c = v - el * NIN;
-        const int e = e0 + el;
-        float xv = 0.0f;
-        if (e < nel) {
-            const int j = e / nlon, i = e - j * nlon;
-            const int s = c / PER, q = c - s * PER;
-            const int nb = s == 0   ? e
-                           : s == 1 ? j * nlon + (i + nlon - 1) % nlon
-                           : s == 2 ? j * nlon + (i + 1) % nlon
-                           : s == 3 ? (j > 0 ? e - nlon : -1)
-                                    : (j < nlat - 1 ? e + nlon : -1);
-            float val = 0.0f;
-            if (nb >= 0) {
+    constexpr int NIN = 60, NOUT = 12, PER = 12, LD = (S / 4) % 2 ? S : S + 4, NT = 8 * S;
+    constexpr int OB1 = FH * NIN, OB2 = OB1 + FH + FH * FH, OB3 = OB2 + FH + NOUT * FH;
+    extern __shared__ __align__(16) float fsm[];
+    __shared__ double red[2 * S];
+    float *const W1 = fsm, *const W2 = W1 + NIN * FH, *const W3 = W2 + FH * FH;
+    float *const X = W3 + FH * FOUT, *const A1 = X + NIN * LD, *const A2 = A1 + FH * LD;
+    const int tid = threadIdx.x;
+    const int s = 4 * (tid % (S / 4)), u = 4 * (tid / (S / 4));
+    const int nel = nlon * nlat, e0 = blockIdx.x * S, ne = min(S, nel - e0);
+    fused_load<NT>(W1, wt + T_W1, NIN * FH);
+    fused_load<NT>(W2, wt + T_W2T, FH * FH);
+    fused_load<NT>(W3, wt + T_W3T, FH * FOUT);
+    dgk::pdl_wait();
+    {   // normalised inputs, the loads of a thread in flight together
+        constexpr int IT = (S * NIN + NT - 1) / NT;
+        float xv[IT], dv[IT], mv[IT], sv[IT];
+#pragma unroll
+        for (int r = 0; r < IT; ++r) {
+            const int v = tid + r * NT, el = v / NIN, c = v - el * NIN, e = e0 + el;
+            const int j = e / nlon, i = e - j * nlon, nbr = c / PER, q = c - nbr * PER;
+            const int nb = nbr == 0   ? e
+                           : nbr == 1 ? (i > 0 ? e - 1 : e + nlon - 1)
+                           : nbr == 2 ? (i < nlon - 1 ? e + 1 : e + 1 - nlon)
+                           : nbr == 3 ? (j > 0 ? e - nlon : -1)
+                                      : (j < nlat - 1 ? e + nlon : -1);
+            xv[r] = dv[r] = 0.0f;
+            mv[r] = __ldg(norm + c);
+            sv[r] = __ldg(norm + NIN + c);
+            if (v < S * NIN && el < ne && nb >= 0) {
                 const size_t o = (size_t)nb * PER + q;
-                val = base[o] + (inc ? inc[o] : 0.0f) + (q == 0 ? 2.0f * href : 0.0f);
+                xv[r] = base[o];
+                dv[r] = (inc ? inc[o] : 0.0f);
+                if (q == 0) mv[r] -= 2.0f * href;   // (mode 0 of h is stored relative to href)
             }
-            xv = (val - norm[c]) / norm[NIN + c];
         }
-        xs[el][c] = xv;
+#pragma unroll
+        for (int r = 0; r < IT; ++r) {
+            const int v = tid + r * NT, el = v / NIN, c = v - el * NIN;
+            if (v < S * NIN) X[c * LD + el] = el < ne ? ((xv[r] + dv[r]) - mv[r]) / sv[r] : 0.0f;
+        }
     }
     __syncthreads();
-    {   // first hidden layer, unit t
-        float z[EPC];
-        const float b = wf[ob1 + t];
-#pragma unroll
-        for (int el = 0; el < EPC; ++el) z[el] = b;
-        for (int c = 0; c < NIN; ++c) {
-            const float w = __bfloat162float(wb[(size_t)t * NIN + c]);
-#pragma unroll
-            for (int el = 0; el < EPC; ++el) z[el] = fmaf(w, xs[el][c], z[el]);
-        }
-#pragma unroll
-        for (int el = 0; el < EPC; ++el) hs[el][t] = gelu(z[el]);
+    float acc[4][4];
+    fused_gemm<LD>(X, W1, NIN, s, u, acc);
+    fused_gelu<LD, false>(acc, wf + OB1, s, u, A1, nullptr);
+    __syncthreads();
+    fused_gemm<LD>(A1, W2, FH, s, u, acc);
+    fused_gelu<LD, false>(acc, wf + OB2, s, u, A2, nullptr);
+    if (tid < 2 * S) red[tid] = 0.0;
+    __syncthreads();
+    for (int v = tid; v < S * NOUT; v += NT) {   // output q of element el
+        const int q = v / S, el = v - q * S, e = e0 + el;
+        if (el >= ne) continue;
+        float y = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < FH; ++k) y = fmaf(A2[k * LD + el], W3[k * FOUT + q], y);
+        y += wf[OB3 + q];
+        // denormalise: per latitude row if row statistics are set, else globally
+        const int j = e / nlon;
+        const float om = rownorm ? rownorm[(size_t)j * NOUT + q] : norm[2 * NIN + q];
+        const float os = rownorm ? rownorm[(size_t)(nlat + j) * NOUT + q] : norm[2 * NIN + NOUT + q];
+        const float out = y * os + om;
+        src[(size_t)e * PER + q] = out;
+        if (q == 0 || q == 2) red[q / 2 * S + el] = c0[j * 2 + q / 2] * (double)out;
     }
     __syncthreads();
-    float a2[EPC];
-    {   // second hidden layer, unit t
-        const float b = wf[ob2 + t];
-#pragma unroll
-        for (int el = 0; el < EPC; ++el) a2[el] = b;
-        for (int c = 0; c < H; ++c) {
-            const float w = __bfloat162float(wb[oW2 + (size_t)t * H + c]);
-#pragma unroll
-            for (int el = 0; el < EPC; ++el) a2[el] = fmaf(w, hs[el][c], a2[el]);
-        }
-#pragma unroll
-        for (int el = 0; el < EPC; ++el) a2[el] = gelu(a2[el]);
+    if (tid < 32) {
+        double m = 0.0;
+        for (int v = tid; v < 2 * S; v += 32) m += red[v];
+        for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        if (tid == 0) part[blockIdx.x] = m;
     }
-    __syncthreads();   // every thread has read the first layer's activations
-#pragma unroll
-    for (int el = 0; el < EPC; ++el) hs[el][t] = a2[el];
-    __syncthreads();
-    if (t < EPC * NOUT) {   // output q of element el
-        const int el = t / NOUT, q = t - el * NOUT;
-        const int e = e0 + el;
-        if (e < nel) {
-            float y = wf[ob3 + q];
-            for (int c = 0; c < H; ++c) y = fmaf(__bfloat162float(wb[oW3 + (size_t)q * H + c]), hs[el][c], y);
-            // denormalise: per latitude row if row statistics are set, else globally
-            const int j = e / nlon;
-            const float om = rownorm ? rownorm[(size_t)j * NOUT + q] : norm[2 * NIN + q];
-            const float os = rownorm ? rownorm[(size_t)(nlat + j) * NOUT + q] : norm[2 * NIN + NOUT + q];
-            src[(size_t)e * PER + q] = y * os + om;
-        }
-    }
+    dgk::pdl_launch_dependents();
 }
 
-// Keep the total mass: remove from mode (a=0, b=0) of h the mass the learned
-// source would add, sum_e sum_b w_j[b] s_e(h, a=0, b) with w_j[b] the mass
-// weights C_j[0][b] of the element's row, spread over the area sum_e w_j[0].
-__global__ void mlp_massfix_kernel(float *__restrict__ src, const double *__restrict__ c0, int nlon, int nlat)
+template <int S>
+int launch_source(const dg_mlp_ctx *m, const float *base, const float *inc, float href, int nlon, int nlat, const double *c0,
+                  float *src, double *part, cudaStream_t s)
 {
-    __shared__ double red[2][256];
-    double m = 0.0, area = 0.0;
-    const int nel = nlon * nlat;
-    for (int e = threadIdx.x; e < nel; e += blockDim.x) {
-        const int j = e / nlon;
-        m += c0[j * 2 + 0] * (double)src[(size_t)e * 12 + 0] + c0[j * 2 + 1] * (double)src[(size_t)e * 12 + 2];
-        area += c0[j * 2 + 0];
+    constexpr int LD = (S / 4) % 2 ? S : S + 4;
+    constexpr size_t bytes = sizeof(float) * (60 * FH + FH * FH + FH * FOUT + (60 + 2 * FH) * LD);
+    static_assert(bytes <= 220 * 1024, "shared memory of one block");
+    static std::atomic<unsigned long long> attr_set{0};   // per device; handles on other host threads may launch too
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    if (!(attr_set.load(std::memory_order_acquire) >> dev & 1ull)) {
+        if (cudaFuncSetAttribute(mlp_source_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return 1;
+        attr_set.fetch_or(1ull << dev, std::memory_order_release);   // setting it twice is harmless
     }
-    red[0][threadIdx.x] = m;
-    red[1][threadIdx.x] = area;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            red[0][threadIdx.x] += red[0][threadIdx.x + s];
-            red[1][threadIdx.x] += red[1][threadIdx.x + s];
-        }
-        __syncthreads();
-    }
-    const float shift = (float)(red[0][0] / red[1][0]);
-    for (int e = threadIdx.x; e < nel; e += blockDim.x) src[(size_t)e * 12] -= shift;
+    const int blocks = (nlon * nlat + S - 1) / S;
+    if (dgk::launch_pdl(mlp_source_kernel<S>, dim3(blocks), dim3(8 * S), bytes, s, base, inc, href, nlon, nlat,
+                        (const __nv_bfloat16 *)m->wt, (const float *)m->w, (const float *)m->norm, (const float *)m->rownorm, c0, src,
+                        part) != cudaSuccess)
+        return 1;
+    return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
+}
+
+// elements of a source block for a mesh of nel elements
+int source_size(int nel)
+{
+    for (int s : {8, 12, 20})
+        if (nel <= 152 * s) return s;
+    return 32;
 }
 
 }  // namespace
 
+int dg_mlp_source_blocks(int nel) { return (nel + source_size(nel) - 1) / source_size(nel); }
+
 int dg_mlp_launch_source(const dg_mlp_ctx *m, const float *base, const float *inc, float href, int nlon, int nlat,
-                         const double *c0, float *src, void *stream)
+                         const double *c0, float *src, double *part, void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int nel = nlon * nlat;
     if (m->rownorm && m->rownorm_nlat != nlat) return 2;   // row statistics of another mesh
-    mlp_source_kernel<<<(nel + SRC_EPC - 1) / SRC_EPC, 128, 0, s>>>(base, inc, href, nlon, nlat, m->wb, m->w, m->ob1, m->oW2, m->ob2,
-                                                     m->oW3, m->ob3, m->norm, m->rownorm, src);
-    mlp_massfix_kernel<<<1, 256, 0, s>>>(src, c0, nlon, nlat);
-    return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
+    switch (source_size(nlon * nlat)) {
+    case 8: return launch_source<8>(m, base, inc, href, nlon, nlat, c0, src, part, s);
+    case 12: return launch_source<12>(m, base, inc, href, nlon, nlat, c0, src, part, s);
+    case 20: return launch_source<20>(m, base, inc, href, nlon, nlat, c0, src, part, s);
+    default: return launch_source<32>(m, base, inc, href, nlon, nlat, c0, src, part, s);
+    }
 }
 
 bool dg_mlp_shape_is(const dg_mlp_ctx *m, int nin, int h, int nout)

@@ -522,6 +522,7 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
     {
         const float cdt = A.cc * A.dt, adt = A.ca * A.dt;
         float chk = 0.f;   // non-finite tendency or state: NaN (nf_acc)
+        const float shift = N == 2 && A.src ? source_shift(A) : 0.f;
         // u^{n+1} = (base + lo) + delta with an error-free two-sum, so
         // increments far below one ulp of the state survive
         auto two_sum = [&](float2 delta, float2 bs, float2 lo, float2 &ob, float2 &ol) {
@@ -572,7 +573,8 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
                     const long long at = at0 + 128 * t;
                     float4 kv = *reinterpret_cast<const float4 *>(M + r * ROW + blk_at(c));
                     if (A.src) {
-                        const float4 s4 = ept_ld4(A.src + at);
+                        float4 s4 = ept_ld4(A.src + at);
+                        if (N == 2 && c % 3 == 0) s4.x -= shift;   // mode 0 of h (an element is three blocks)
                         kv.x += s4.x, kv.y += s4.y, kv.z += s4.z, kv.w += s4.w;
                     }
                     if (VEC || (4 * c >= ld && 4 * c + 4 <= end)) {
