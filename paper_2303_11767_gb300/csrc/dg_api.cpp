@@ -410,6 +410,7 @@ template <typename T>
 dg_status upload_rows(dg_ctx *h, RowTab<T> **dst)
 {
     std::vector<RowTab<T>> r(h->nlat);
+    const StageArgs<double> mesh = base_args<double>(h, nullptr, 0.0);
     for (int j = 0; j < h->nlat; ++j) {
         const RowTab<double> &s = h->tab.rows[j];
         RowTab<T> &d = r[j];
@@ -418,6 +419,9 @@ dg_status upload_rows(dg_ctx *h, RowTab<T> **dst)
             d.cosn[a] = (T)s.cosn[a];
             d.sinn[a] = (T)s.sinn[a];
             d.rho[a] = (T)s.rho[a];
+            d.cGc[a] = (T)(mesh.cG * s.cosn[a]);
+            d.sR[a] = (T)(s.sinn[a] * mesh.invR);
+            d.fc[a] = (T)(mesh.twoOmega * s.sinn[a] * s.cosn[a]);
             d.CSE[a] = (T)s.CSE[a];
             d.CSW[a] = (T)s.CSW[a];
             for (int b = 0; b < DG_MAXN; ++b) {

@@ -35,8 +35,26 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 
 template <typename T>
 __device__ __forceinline__ T rcp(T x);
+// FP64: the FP64 pipe (2 lanes per SM) bounds the FP64 stage, and a division
+// or square root takes 9 to 14 of its operations.  Within a range that holds
+// every depth, 1 / x and sqrt(x) are the hardware's approximation (relative
+// residual e below 2^-19) with one third-order correction from the binomial
+// series, (1 - e)^-1 = 1 + e + e^2 + .. and (1 - e)^-1/2 = 1 + e/2 + 3 e^2/8 +
+// .., whose remainder is below 2^-56: 3 and 5 operations, and within one ulp
+// (0.5 before).  Other arguments take the division and sqrt().
+__device__ __forceinline__ bool plain_range(double x)   // 2^-900 < x < 2^900, from the exponent
+{
+    return (unsigned)(__double2hiint(x) - 0x07b00000) < 0x70800000u;
+}
 template <>
-__device__ __forceinline__ double rcp<double>(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp<double>(double x)
+{
+    if (!plain_range(x)) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
 // FP32: the SFU reciprocal alone (<= 1 ulp; __fdividef(1, x) scales its
 // argument around it, for depths that do not occur)
 template <>
@@ -50,7 +68,14 @@ __device__ __forceinline__ float rcp<float>(float x)
 template <typename T>
 __device__ __forceinline__ T wave_sqrt(T x);
 template <>
-__device__ __forceinline__ double wave_sqrt<double>(double x) { return sqrt(x); }
+__device__ __forceinline__ double wave_sqrt<double>(double x)
+{
+    if (!plain_range(x)) return sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double s = x * y, e = fma(-s, y, 1.0);
+    return fma(s * e, fma(0.375, e, 0.5), s);
+}
 // FP32: x * rsqrt(x) on the SFU; only feeds the Rusanov dissipation speed
 template <>
 __device__ __forceinline__ float wave_sqrt<float>(float x)
@@ -68,6 +93,11 @@ __device__ __forceinline__ float wave_sqrt<float>(float x)
 __device__ __forceinline__ float nf_acc(float x, float chk) { return __fmaf_rn(x, 0.0f, chk); }
 __device__ __forceinline__ double nf_acc(double x, double chk) { return __fma_rn(x, 0.0, chk); }
 
+// The same for FP64 with integer operations on the exponent, off the FP64
+// pipe: the largest magnitude word seen.
+__device__ __forceinline__ unsigned nf_acc_bits(double x, unsigned m) { return max(m, (unsigned)__double2hiint(x) & 0x7fffffffu); }
+__device__ __forceinline__ bool nf_bits(unsigned m) { return m >= 0x7ff00000u; }
+
 // h <= 0 makes u = hu/h meaningless; a NaN depth is reported as non-finite.
 template <typename T>
 __device__ __forceinline__ void check_depth(T h, unsigned &st)
@@ -75,10 +105,41 @@ __device__ __forceinline__ void check_depth(T h, unsigned &st)
     if (!(h > T(0))) st |= (h != h) ? DG_STATUS_NONFINITE : DG_STATUS_NONPHYSICAL;
 }
 
+// (FP64: the compares only where the exponent is not that of a positive number)
+template <>
+__device__ __forceinline__ void check_depth<double>(double h, unsigned &st)
+{
+    if ((unsigned)(__double2hiint(h) - 1) >= 0x7fefffffu && !(h > 0.0))
+        st |= (h != h) ? DG_STATUS_NONFINITE : DG_STATUS_NONPHYSICAL;
+}
+
 // Every multiply-add below is an explicit fma: these functions are inlined at
 // several call sites (an edge's flux is evaluated by whichever tile or band
 // owns it), and left to the compiler's contraction the same edge could round
 // differently at two sites.
+
+// P = g h' (href + h'/2); FP64 with the constants folded, one operation less
+template <typename T>
+__device__ __forceinline__ T pressure(T hp, T href, T g) { return (hp * g) * fma(T(0.5), hp, href); }
+template <>
+__device__ __forceinline__ double pressure<double>(double hp, double href, double g) { return hp * fma(0.5 * g, hp, g * href); }
+
+// out = c/2 ((fl + fr) - a (R - L)), a the larger of the speeds (both >= 0)
+template <typename T>
+__device__ __forceinline__ void rusanov_out(const T *L, const T *R, const T *fl, const T *fr, T al, T ar, T aglob, T c, T *out)
+{
+    if constexpr (sizeof(T) == 8) {
+        // non-negative doubles order like their bits; the factor 1/2 sits in c
+        const double a = aglob > 0.0 ? aglob : __longlong_as_double(max(__double_as_longlong(al), __double_as_longlong(ar)));
+        const double hc = 0.5 * c;
+#pragma unroll
+        for (int f = 0; f < 3; ++f) out[f] = hc * fma(-a, R[f] - L[f], __dadd_rn(fl[f], fr[f]));
+    } else {
+        const T ha = T(0.5) * (aglob > T(0) ? aglob : fmax(al, ar));   // global mode: the stage's largest |u| + c
+#pragma unroll
+        for (int f = 0; f < 3; ++f) out[f] = c * fma(-ha, R[f] - L[f], T(0.5) * (fl[f] + fr[f]));
+    }
+}
 
 // Physical lambda-flux (hu, hu u + P, hu v) of a state q = (h', hu, hv) with
 // h = href + h' and the pressure P = g h' (href + h'/2) (the constant part
@@ -89,7 +150,7 @@ __device__ __forceinline__ void lam_flux(const T *q, T href, T g, T *f, T &speed
     const T h = href + q[0];
     check_depth(h, st);
     const T u = q[1] * rcp(h);
-    const T P = (q[0] * g) * fma(T(0.5), q[0], href);
+    const T P = pressure(q[0], href, g);
     f[0] = q[1];
     f[1] = fma(q[1], u, P);
     f[2] = q[2] * u;
@@ -102,7 +163,7 @@ __device__ __forceinline__ void th_flux(const T *q, T href, T g, T *f, T &speed,
     const T h = href + q[0];
     check_depth(h, st);
     const T v = q[2] * rcp(h);
-    const T P = (q[0] * g) * fma(T(0.5), q[0], href);
+    const T P = pressure(q[0], href, g);
     f[0] = q[2];
     f[1] = q[1] * v;
     f[2] = fma(q[2], v, P);
@@ -120,9 +181,7 @@ __device__ __forceinline__ void rusanov_lam(const T *L, const T *R, T href, T g,
     T fl[3], fr[3], al, ar;
     lam_flux(L, href, g, fl, al, st);
     lam_flux(R, href, g, fr, ar, st);
-    const T ha = T(0.5) * (aglob > T(0) ? aglob : fmax(al, ar));   // global mode: the stage's largest |u| + c
-#pragma unroll
-    for (int f = 0; f < 3; ++f) out[f] = cF * fma(-ha, R[f] - L[f], T(0.5) * (fl[f] + fr[f]));
+    rusanov_out(L, R, fl, fr, al, ar, aglob, cF, out);
 }
 
 // Rusanov flux through a theta-face, lower state S, upper state N, times the
@@ -134,9 +193,7 @@ __device__ __forceinline__ void rusanov_th(const T *S, const T *Nq, T href, T g,
     T fs[3], fn[3], as, an;
     th_flux(S, href, g, fs, as, st);
     th_flux(Nq, href, g, fn, an, st);
-    const T ha = T(0.5) * (aglob > T(0) ? aglob : fmax(as, an));   // global mode: the stage's largest |v| + c
-#pragma unroll
-    for (int f = 0; f < 3; ++f) out[f] = cGce * fma(-ha, Nq[f] - S[f], T(0.5) * (fs[f] + fn[f]));
+    rusanov_out(S, Nq, fs, fn, as, an, aglob, cGce, out);
 }
 
 }  // namespace dgk

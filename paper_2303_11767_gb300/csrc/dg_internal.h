@@ -29,6 +29,8 @@ struct BasisTab {
 //   CSE, CSW: Ci * L(+1), Ci * L(-1) (north / south lift)
 //   rho: hv tendency of the (a = 0, b) modes produced by a unit constant
 //        pressure flux (the rest state with g h^2 / 2 = 1), n-point rules
+//   cGc, sR, fc: cG cos, sin / R and 2 Omega sin cos at the Gauss points, the
+//        row constants of the FP64 stage's pointwise phase (filled at upload)
 template <typename T>
 struct RowTab {
     T cosn[DG_MAXN];
@@ -41,6 +43,7 @@ struct RowTab {
     T CSE[DG_MAXN];
     T CSW[DG_MAXN];
     T rho[DG_MAXN];
+    T cGc[DG_MAXN], sR[DG_MAXN], fc[DG_MAXN];
 };
 
 // Host-side FP64 tables of one mesh.
