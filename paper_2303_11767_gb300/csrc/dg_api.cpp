@@ -300,7 +300,7 @@ dg_status enqueue_source(dg_ctx *h, StageArgs<float> &a)
     a.src_parts = dg_mlp_source_blocks((int)h->nel);
     double area = 0.0;   // sum over the elements of the mass weight of mode 0
     for (int j = 0; j < h->nlat; ++j) area += h->tab.C[(size_t)j * h->nphi];
-    a.src_area = area * h->nlon;
+    a.src_rarea = 1.0 / (area * h->nlon);
     h->aux_launches += 1;
     return DG_OK;
 }

@@ -89,10 +89,10 @@ struct StageArgs {
     T *out_base;
     T *out_lo;
     const T *src;    // optional modal source added to k (learned correction), after
-                     // (sum of src_part[0 .. src_parts)) / src_area is taken from mode 0 of h
+                     // (sum of src_part[0 .. src_parts)) * src_rarea is taken from mode 0 of h
     const double *src_part;
     int src_parts;
-    double src_area;
+    double src_rarea;
     const T *galpha; // global Rusanov mode: [max |u| + c, max |v| + c] of the stage input; null = local
     const RowTab<T> *rows;
     unsigned int *status;

@@ -323,15 +323,16 @@ __device__ __forceinline__ void load_stage_row(const T *__restrict__ base, const
 }
 
 // What is taken from mode 0 of h of the learned source so that it adds no
-// mass: the blocks' sums over the area, in a fixed order (every warp forms it
-// for itself).
+// mass: the blocks' sums over the area, in a fixed order, by one whole warp.
+// The stage forms it at its start, while the other warps load the tile (a
+// dependent FP64 operation takes about 50 ns).
 template <typename T>
 __device__ __forceinline__ T source_shift(const StageArgs<T> &A)
 {
     double m = 0.0;
     for (int v = threadIdx.x & 31; v < A.src_parts; v += 32) m += A.src_part[v];
     for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-    return (T)(m / A.src_area);
+    return (T)(m * A.src_rarea);
 }
 
 // One tile of G x W elements (tile column bx, tile row by) of one mesh.  The
@@ -376,6 +377,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
 
     const RowTab<T> *RT = A.rows + (valid ? j : 0);
     const T ga_l = A.galpha ? A.galpha[0] : T(0), ga_t = A.galpha ? A.galpha[1] : T(0);
+
+    __shared__ T src_shift;   // (read after the tile's barriers)
+    if (N == 2 && A.src && warp == W - 1) {
+        const T v = source_shift(A);
+        if (lane == 0) src_shift = v;
+    }
 
     // ---- S0: own modal row b = k of the stage state
     T uh[3][N];
@@ -954,7 +961,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
             }
         }
         kk[2][0] = fma(A.P0, rhok, kk[2][0]);
-        const T shift = N == 2 && A.src ? source_shift(A) : T(0);
+        const T shift = N == 2 && A.src ? src_shift : T(0);
         if (A.src && valid) {   // learned modal source, same layout as the state
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
@@ -1223,7 +1230,7 @@ __global__ void __launch_bounds__(32 * W, 24 / W) ensemble_kernel(const EnsArgs<
         A.src = nullptr;
         A.src_part = nullptr;
         A.src_parts = 0;
-        A.src_area = 0;
+        A.src_rarea = 0;
         A.galpha = nullptr;
         A.status = E.status;
         A.nlon = m.nlon;

@@ -583,11 +583,13 @@ dg_status dg_mlp_train_step(dg_mlp m, const float *d_x, const float *d_t, int ba
 
 namespace {
 
-// Block of 8 S threads: the network for S consecutive elements of a degree-1
+// Block of 32 S threads: the network for S consecutive elements of a degree-1
 // mesh.  It gathers each element's and its four neighbours' modes (zeros
-// across a pole), normalises them into shared memory and runs the layers as
-// the training kernel does (4 elements x 4 units of a layer per thread, k-major
-// weights).  The state is u_stage = base + inc with h stored relative to href
+// across a pole), normalises them into shared memory and runs the layers on
+// tiles of 4 elements x 4 units per thread with k-major weights, as the
+// training kernel does; four groups of threads share a layer's inputs and add
+// their sums through shared memory (with one group an SM had 5 warps, 18 % of
+// the issue slots: 21.9 us per stage, source and stage together, against 15.2).  The state is u_stage = base + inc with h stored relative to href
 // (mode 0 of h carries 2 href).  The mass that the source would add,
 // sum_b w_j[b] s(h, a = 0, b) with w_j[b] the mass weights C_j[0][b] of the
 // element's row, is summed over the block into part: the stage kernel removes
@@ -596,22 +598,52 @@ namespace {
 // The weights (51 KB) are read once per block before the wait for the previous
 // stage, so S is the smallest size that gives every SM at most one block.  At
 // 72x36, per stage: one thread per hidden unit reading its own weight row 46 us
-// and a single-block mass sum 13 us; now 15 us together.
+// and a single-block mass sum 13 us; now 15 us with the stage.
+constexpr int SRC_KS = 4;
+
+// One hidden layer of the source block: A -> gelu(A W + b) (K inputs), the
+// groups' partial sums in P [group][unit][LD]
+template <int S, int LD, int K>
+__device__ __forceinline__ void source_layer(const float *A, const float *W, const float *__restrict__ bias, float *P, float *out)
+{
+    constexpr int T1 = 8 * S, KG = K / SRC_KS;
+    static_assert(K % SRC_KS == 0, "equal groups");
+    const int tid = threadIdx.x, ks = tid / T1, t = tid - ks * T1;
+    const int s = 4 * (t % (S / 4)), u = 4 * (t / (S / 4));
+    float acc[4][4];
+    fused_gemm<LD>(A + ks * KG * LD, W + ks * KG * FH, KG, s, u, acc);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<float4 *>(P + (ks * FH + u + j) * LD + s) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+    __syncthreads();
+    const int un = u + ks;   // a quarter of the tile's units each
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int g = 0; g < SRC_KS; ++g) {
+        const float4 v = *reinterpret_cast<const float4 *>(P + (g * FH + un) * LD + s);
+        z[0] += v.x, z[1] += v.y, z[2] += v.z, z[3] += v.w;
+    }
+    const float b = __ldg(bias + un);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) z[i] = gelu(z[i] + b);
+    *reinterpret_cast<float4 *>(out + un * LD + s) = make_float4(z[0], z[1], z[2], z[3]);
+    __syncthreads();
+}
+
 template <int S>
-__global__ void __launch_bounds__(8 * S) mlp_source_kernel(const float *__restrict__ base, const float *__restrict__ inc, float href,
+__global__ void __launch_bounds__(8 * S * SRC_KS) mlp_source_kernel(const float *__restrict__ base, const float *__restrict__ inc, float href,
                                                            int nlon, int nlat, const __nv_bfloat16 *__restrict__ wt,
                                                            const float *__restrict__ wf, const float *__restrict__ norm,
                                                            const float *__restrict__ rownorm, const double *__restrict__ c0,
                                                            float *__restrict__ src, double *__restrict__ part)
 {
-    constexpr int NIN = 60, NOUT = 12, PER = 12, LD = (S / 4) % 2 ? S : S + 4, NT = 8 * S;
+    constexpr int NIN = 60, NOUT = 12, PER = 12, LD = (S / 4) % 2 ? S : S + 4, NT = 8 * S * SRC_KS;
     constexpr int OB1 = FH * NIN, OB2 = OB1 + FH + FH * FH, OB3 = OB2 + FH + NOUT * FH;
     extern __shared__ __align__(16) float fsm[];
     __shared__ double red[2 * S];
     float *const W1 = fsm, *const W2 = W1 + NIN * FH, *const W3 = W2 + FH * FH;
-    float *const X = W3 + FH * FOUT, *const A1 = X + NIN * LD, *const A2 = A1 + FH * LD;
+    float *const X = W3 + FH * FOUT, *const A1 = X + NIN * LD, *const A2 = A1 + FH * LD, *const P = A2 + FH * LD;
     const int tid = threadIdx.x;
-    const int s = 4 * (tid % (S / 4)), u = 4 * (tid / (S / 4));
     const int nel = nlon * nlat, e0 = blockIdx.x * S, ne = min(S, nel - e0);
     fused_load<NT>(W1, wt + T_W1, NIN * FH);
     fused_load<NT>(W2, wt + T_W2T, FH * FH);
@@ -646,20 +678,17 @@ __global__ void __launch_bounds__(8 * S) mlp_source_kernel(const float *__restri
         }
     }
     __syncthreads();
-    float acc[4][4];
-    fused_gemm<LD>(X, W1, NIN, s, u, acc);
-    fused_gelu<LD, false>(acc, wf + OB1, s, u, A1, nullptr);
-    __syncthreads();
-    fused_gemm<LD>(A1, W2, FH, s, u, acc);
-    fused_gelu<LD, false>(acc, wf + OB2, s, u, A2, nullptr);
+    source_layer<S, LD, NIN>(X, W1, wf + OB1, P, A1);
     if (tid < 2 * S) red[tid] = 0.0;
-    __syncthreads();
-    for (int v = tid; v < S * NOUT; v += NT) {   // output q of element el
-        const int q = v / S, el = v - q * S, e = e0 + el;
-        if (el >= ne) continue;
+    source_layer<S, LD, FH>(A1, W2, wf + OB2, P, A2);
+    // output q of element el by a pair of lanes, even and odd units
+    for (int v = tid; v < (2 * S * NOUT + 31) / 32 * 32; v += NT) {   // whole warps
+        const int o = min(v >> 1, S * NOUT - 1), h = v & 1, q = o / S, el = o - q * S, e = e0 + el;
         float y = 0.f;
 #pragma unroll 8
-        for (int k = 0; k < FH; ++k) y = fmaf(A2[k * LD + el], W3[k * FOUT + q], y);
+        for (int k = h; k < FH; k += 2) y = fmaf(A2[k * LD + el], W3[k * FOUT + q], y);
+        y += __shfl_xor_sync(0xffffffffu, y, 1);
+        if (h || el >= ne || v >= 2 * S * NOUT) continue;
         y += wf[OB3 + q];
         // denormalise: per latitude row if row statistics are set, else globally
         const int j = e / nlon;
@@ -684,8 +713,8 @@ int launch_source(const dg_mlp_ctx *m, const float *base, const float *inc, floa
                   float *src, double *part, cudaStream_t s)
 {
     constexpr int LD = (S / 4) % 2 ? S : S + 4;
-    constexpr size_t bytes = sizeof(float) * (60 * FH + FH * FH + FH * FOUT + (60 + 2 * FH) * LD);
-    static_assert(bytes <= 220 * 1024, "shared memory of one block");
+    constexpr size_t bytes = sizeof(float) * (60 * FH + FH * FH + FH * FOUT + (60 + (2 + SRC_KS) * FH) * LD);
+    static_assert(bytes <= 226 * 1024, "shared memory of one block");
     static std::atomic<unsigned long long> attr_set{0};   // per device; handles on other host threads may launch too
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
@@ -694,7 +723,7 @@ int launch_source(const dg_mlp_ctx *m, const float *base, const float *inc, floa
         attr_set.fetch_or(1ull << dev, std::memory_order_release);   // setting it twice is harmless
     }
     const int blocks = (nlon * nlat + S - 1) / S;
-    if (dgk::launch_pdl(mlp_source_kernel<S>, dim3(blocks), dim3(8 * S), bytes, s, base, inc, href, nlon, nlat,
+    if (dgk::launch_pdl(mlp_source_kernel<S>, dim3(blocks), dim3(8 * S * SRC_KS), bytes, s, base, inc, href, nlon, nlat,
                         (const __nv_bfloat16 *)m->wt, (const float *)m->w, (const float *)m->norm, (const float *)m->rownorm, c0, src,
                         part) != cudaSuccess)
         return 1;

@@ -248,6 +248,12 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
     unsigned st = 0;
     float hmin = INFINITY;   // smallest depth at the Gauss points
 
+    __shared__ float src_shift;   // (read after the tile's barriers)
+    if (N == 2 && A.src && warp == NT / 32 - 1) {
+        const float v = source_shift(A);
+        if (lane == 0) src_shift = v;
+    }
+
     // ---- S0: the tile's stage state, flat 16-byte blocks, each warp its rows.
     // Block c of a row holds the values 4 c - lead .. of its segment.
     auto row_off = [&](int jj) -> long long { return ((long long)jj * A.nlon + i0) * EL; };
@@ -522,7 +528,7 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
     {
         const float cdt = A.cc * A.dt, adt = A.ca * A.dt;
         float chk = 0.f;   // non-finite tendency or state: NaN (nf_acc)
-        const float shift = N == 2 && A.src ? source_shift(A) : 0.f;
+        const float shift = N == 2 && A.src ? src_shift : 0.f;
         // u^{n+1} = (base + lo) + delta with an error-free two-sum, so
         // increments far below one ulp of the state survive
         auto two_sum = [&](float2 delta, float2 bs, float2 lo, float2 &ob, float2 &ol) {
