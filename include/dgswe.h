@@ -199,7 +199,10 @@ dg_status dg_projection_nodes(dg_handle h, double *lam, size_t nlam, double *the
  * onto the modal basis.  nodal holds the three fields at the projection
  * points of every element, layout [j][i][f][q_theta][q_lambda]
  * (len_nodal = nlat * nlon * 3 * nm * nm); modal_out receives dg_state_len(h)
- * values.  Host computation in FP64; does not touch the resident state. */
+ * values.  Computed in FP64 on the GPU, in portions of 32 MB through a workspace
+ * that the handle keeps (on the host where there is no memory for it or the
+ * solver's stream is being captured); synchronises the solver's stream and
+ * does not touch the resident state. */
 dg_status dg_project_nodal(dg_handle h, const double *nodal, size_t len_nodal, double *modal_out,
                            size_t len);
 

@@ -86,6 +86,8 @@ struct dg_ctx {
     void *SL[2] = {nullptr, nullptr};
     int cur = 0;                       // index of B / L holding u^n
     double *stage64 = nullptr;                            // FP64 staging of one state
+    double *proj = nullptr;                               // projection workspace: tables, then point values
+    size_t proj_tab = 0, proj_vals = 0;                   // values of each
     RowTab<double> *rows64 = nullptr;
     RowTab<float> *rows32 = nullptr;
     double *c0 = nullptr;                                 // mass table: C_j[0][b], then row areas
@@ -718,6 +720,7 @@ dg_status dg_destroy(dg_handle h)
     drop_graphs(h);
     free_state_buffers(h);
     cudaFree(h->stage64);
+    cudaFree(h->proj);
     cudaFree(h->rows64);
     cudaFree(h->rows32);
     cudaFree(h->c0);
@@ -1206,6 +1209,69 @@ dg_status dg_projection_nodes(dg_handle h, double *lam, size_t nlam, double *the
     return DG_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+constexpr size_t PROJ_BYTES = 32u << 20;   // point values held on the device at a time
+
+// The projection on the GPU, in portions of PROJ_BYTES through a workspace that
+// the handle keeps; *done stays false where it cannot be had (no memory, or
+// the stream is being captured) and nothing has been written.
+dg_status project_on_device(dg_ctx *h, const double *nodal, double *modal_out, const std::vector<double> &PL, bool *done)
+{
+    *done = false;
+    const int n = h->n, nm = h->tab.nm;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return DG_OK;
+    }
+    const size_t nq = (size_t)nm * nm, pairs = h->nel * 3;
+    if (!h->proj) {
+        h->proj_tab = ((size_t)(n + h->nlat) * nm + 31) / 32 * 32;
+        h->proj_vals = std::min(pairs, std::max<size_t>(1, PROJ_BYTES / (sizeof(double) * nq))) * nq;
+        std::vector<double> tab(h->proj_tab, 0.0);
+        std::copy(PL.begin(), PL.end(), tab.begin());
+        for (int j = 0; j < h->nlat; ++j) {
+            const double tb = -0.5 * M_PI + (h->j0 + j) * h->tab.dth;
+            for (int q = 0; q < nm; ++q)
+                tab[(size_t)(n + j) * nm + q] = std::cos(tb + 0.5 * (1.0 + h->tab.xm[q]) * h->tab.dth);
+        }
+        // another thread's stream capture does not forbid this allocation
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const cudaError_t e = cudaMalloc(&h->proj, sizeof(double) * (h->proj_tab + h->proj_vals));
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            h->proj = nullptr;
+            return DG_OK;
+        }
+        if (cudaMemcpyAsync(h->proj, tab.data(), sizeof(double) * h->proj_tab, cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+            cudaStreamSynchronize(h->stream) != cudaSuccess) {
+            cudaFree(h->proj);
+            h->proj = nullptr;
+            return fail(DG_ECUDA, "copy of the projection tables failed");
+        }
+    }
+    *done = true;
+    double *const v = h->proj + h->proj_tab;
+    for (size_t p = 0; p < pairs; p += h->proj_vals / nq) {
+        const size_t np = std::min(pairs - p, h->proj_vals / nq);
+        CUDA_TRY(cudaMemcpyAsync(v, nodal + p * nq, sizeof(double) * np * nq, cudaMemcpyHostToDevice, h->stream));
+        if (dg_launch_project(n, v, p, (int)np, h->nlon, nm, h->proj, h->proj + (size_t)n * nm, h->rows64, h->stage64, h->stream))
+            return fail(DG_ECUDA, "projection kernel failed: %s", cudaGetErrorString(cudaGetLastError()));
+    }
+    CUDA_TRY(cudaMemcpyAsync(modal_out, h->stage64, sizeof(double) * h->len, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    return DG_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 dg_status dg_project_nodal(dg_handle h, const double *nodal, size_t len_nodal, double *modal_out, size_t len)
 {
     if (dg_status s = check(h)) return s;
@@ -1242,6 +1308,13 @@ dg_status dg_project_nodal(dg_handle h, const double *nodal, size_t len_nodal, d
     std::vector<double> PL((size_t)n * nm), PC((size_t)n * nm), s((size_t)nm * n), r((size_t)n * n);
     for (int a = 0; a < n; ++a)
         for (int q = 0; q < nm; ++q) PL[(size_t)a * nm + q] = h->tab.wm[q] * dg_legendre(a, h->tab.xm[q]);
+    {
+        DeviceGuard dg(h->device);
+        bool done = false;
+        if (dg_status st = project_on_device(h, nodal, modal_out, PL, &done)) return st;
+        if (done) return DG_OK;
+    }
+    // the same sums on the host
     for (int j = 0; j < h->nlat; ++j) {
         const double tb = -0.5 * M_PI + (h->j0 + j) * h->tab.dth;
         for (int b = 0; b < n; ++b)

@@ -193,6 +193,11 @@ int dg_launch_max_speed(const T *u, int nlon, int nlat, int n, double href, doub
                         unsigned long long *maxbits, unsigned int *status, void *stream);
 int dg_mass_blocks(size_t nel);
 
+// dg_project.cu: npairs (element, field) pairs from pair0 of a mesh, nm x nm
+// point values each (v), onto its modes; see there for the tables.
+int dg_launch_project(int n, const double *v, size_t pair0, int npairs, int nlon, int nm, const double *pl, const double *cosm,
+                      const RowTab<double> *rows, double *out, void *stream);
+
 // dg_restrict.cu: nested fine -> coarse projection
 struct RestrictTab {
     double x[8], w[8];            // 8-point Gauss rule on [-1, 1]
