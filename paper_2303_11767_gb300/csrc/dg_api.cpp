@@ -95,7 +95,7 @@ struct dg_ctx {
     int nblocks = 0;
     double *d_result = nullptr;
     unsigned *d_status = nullptr;
-    unsigned long long *d_maxbits = nullptr;
+    unsigned long long *d_maxbits = nullptr;              // scratch of the wave-speed maximum
     void *galpha = nullptr;   // global Rusanov mode: the stage's two speeds (2 values of T)
     double href = 0;      // reference depth of the resident state (FP32 path, or well balanced); else 0
     int wb = 0;           // well-balanced option: the rest state at href is exactly steady
@@ -595,7 +595,7 @@ dg_status create_sphere(int nlon, int nlat_g, int jb, int je, int degree, double
     if (cudaMalloc(&h->partials, 2 * sizeof(double) * (h->nblocks + 1)) != cudaSuccess ||   // + the pair
         cudaMalloc(&h->d_result, sizeof(double)) != cudaSuccess ||
         cudaMalloc(&h->d_status, sizeof(unsigned)) != cudaSuccess ||
-        cudaMalloc(&h->d_maxbits, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&h->d_maxbits, 2 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc(&h->galpha, 2 * sizeof(double)) != cudaSuccess) {
         dg_destroy(h);
         return fail(DG_ENOMEM, "cudaMalloc failed");
@@ -1135,12 +1135,11 @@ namespace {
 // Gauss points of sqrt(u^2 + v^2) + sqrt(g h).
 dg_status cfl_terms(dg_ctx *h, double *H_out, double *c_out)
 {
-    CUDA_TRY(cudaMemsetAsync(h->d_maxbits, 0, sizeof(unsigned long long), h->stream));
     int r = h->prec == DG_PREC_FP64
                 ? dg_launch_max_speed<double>(static_cast<const double *>(h->B[h->cur]), h->nlon, h->nlat, h->n,
-                                              h->href, h->g, h->d_maxbits, h->d_status, h->stream)
+                                              h->href, h->g, h->d_maxbits, reinterpret_cast<float *>(h->stage64), h->d_status, h->stream)
                 : dg_launch_max_speed<float>(static_cast<const float *>(h->B[h->cur]), h->nlon, h->nlat, h->n,
-                                             h->href, h->g, h->d_maxbits, h->d_status, h->stream);
+                                             h->href, h->g, h->d_maxbits, reinterpret_cast<float *>(h->stage64), h->d_status, h->stream);
     if (r) return fail(DG_ECUDA, "wave-speed kernel failed: %s", cudaGetErrorString(cudaGetLastError()));
     unsigned long long bits = 0;
     CUDA_TRY(cudaMemcpyAsync(&bits, h->d_maxbits, sizeof bits, cudaMemcpyDeviceToHost, h->stream));

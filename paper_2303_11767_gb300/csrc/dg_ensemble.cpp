@@ -60,7 +60,7 @@ struct dg_ens {
     std::vector<size_t> c0_off;
     int nblocks = 0;
     unsigned *d_status = nullptr;
-    unsigned long long *d_maxbits = nullptr;
+    unsigned long long *d_maxbits = nullptr;   // scratch of the wave-speed maximum
     std::vector<double> href, dt;
     std::vector<char> have;
     int tile_rows = DG_ENS_TILE_ROWS_B, bps = 2, spg = 16;
@@ -295,7 +295,7 @@ dg_status dg_ensemble_create(int members, const int *nlon, const int *nlat, cons
     if (cudaMalloc(&e->partials, 2 * sizeof(double) * e->nblocks) != cudaSuccess ||
         cudaMalloc(&e->d_result, sizeof(double)) != cudaSuccess ||
         cudaMalloc(&e->d_status, sizeof(unsigned)) != cudaSuccess ||
-        cudaMalloc(&e->d_maxbits, sizeof(unsigned long long)) != cudaSuccess)
+        cudaMalloc(&e->d_maxbits, 2 * sizeof(unsigned long long)) != cudaSuccess)
         ETRY(efail(DG_ENOMEM, "cudaMalloc failed"));
     if (cudaMemset(e->d_status, 0, sizeof(unsigned)) != cudaSuccess) ETRY(efail(DG_ECUDA, "cudaMemset failed"));
     // the device table must exist before the first launch
@@ -505,9 +505,8 @@ dg_status dg_ensemble_max_dt(dg_ensemble e, int member, double cfl, double *dt)
     if (dg_status s = check_member(e, member)) return s;
     if (!dt || !(cfl > 0)) return efail(DG_EINVAL, "need cfl > 0 and dt != NULL");
     const int n = e->deg[member] + 1;
-    ECUDA(cudaMemsetAsync(e->d_maxbits, 0, sizeof(unsigned long long), e->stream));
     if (dg_launch_max_speed<float>(e->B[e->cur] + e->off[member], e->nlon[member], e->nlat[member], n,
-                                   e->href[member], e->g, e->d_maxbits, e->d_status, e->stream))
+                                   e->href[member], e->g, e->d_maxbits, reinterpret_cast<float *>(e->stage64), e->d_status, e->stream))
         return efail(DG_ECUDA, "wave-speed kernel failed");
     unsigned long long bits = 0;
     ECUDA(cudaMemcpyAsync(&bits, e->d_maxbits, sizeof bits, cudaMemcpyDeviceToHost, e->stream));

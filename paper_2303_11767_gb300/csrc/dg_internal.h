@@ -188,9 +188,11 @@ int dg_launch_mass(const T *u, const T *lo, const double *c0, int nlon, int nlat
 template <typename T>
 int dg_launch_global_speeds(int n, const T *base, const T *inc, int nlon, int nlat, int lanes, T href, T g, T *out,
                             void *stream);
+// Largest wave speed over the Gauss points, as the bits of a positive double in
+// maxbits[0] (two words of scratch); upper: one float of scratch per element.
 template <typename T>
 int dg_launch_max_speed(const T *u, int nlon, int nlat, int n, double href, double g,
-                        unsigned long long *maxbits, unsigned int *status, void *stream);
+                        unsigned long long *maxbits, float *upper, unsigned int *status, void *stream);
 int dg_mass_blocks(size_t nel);
 
 // dg_project.cu: npairs (element, field) pairs from pair0 of a mesh, nm x nm

@@ -1403,39 +1403,144 @@ static __global__ void __launch_bounds__(MASS_THREADS) mass_final_kernel(const d
     }
 }
 
-// Largest sqrt(u^2 + v^2) + sqrt(g h) over the n x n Gauss points; one thread
-// per element.  Positive doubles order like their bit patterns, so an atomic
-// max on the bits is exact and order independent.
+// Largest sqrt(u^2 + v^2) + sqrt(g h) over the n x n Gauss points, in FP64 and
+// exactly, without evaluating every point in FP64 (about 2300 operations per
+// element at degree 4 on a pipe of 2 lanes per SM: 11 ms at 1440x720).
+// First an FP32 pass bounds every element's speed from above and below; then
+// only the elements whose upper bound reaches the largest lower bound are
+// evaluated in FP64, a warp per element.  The bounds cover the rounding of
+// the FP32 pass: a point value is a sum of N^2 terms |m| |L_a| |L_b|, at most
+// S = sum |m| max|L_a| max|L_b| in size, and carries at most 2 N + 4 < 16
+// roundings, so its error is below 2^-20 S; 2^-19 is used.  A point whose
+// depth is not surely positive, and anything non-finite, goes to the FP64 pass,
+// which reports it.  dg_max_dt at 1440x720 degree 4: 10.0 -> 0.28 ms
+// (a fluid at rest, where every element ties: 11.2 -> 7.3 ms).
+constexpr int SPEED_THREADS = 64;
+
 template <typename T, int N>
-__global__ void max_speed_kernel(const T *__restrict__ u, int nel, double href, double g,
-                                 unsigned long long *maxbits, unsigned *status)
+__global__ void __launch_bounds__(SPEED_THREADS) speed_bound_kernel(const T *__restrict__ u, int nel, float href, float g,
+                                                                    float *__restrict__ upper, unsigned *__restrict__ lower)
+{
+    constexpr int NP = N * N, EL = 3 * NP, ES = EL | 1;   // odd stride: a lane's element in its own bank
+    __shared__ float sm[SPEED_THREADS * ES];
+    const BasisTab<T> &B = c_basis[N - 1];
+    const int e0 = blockIdx.x * SPEED_THREADS, ne = min(SPEED_THREADS, nel - e0);
+    const T *const src = u + (size_t)e0 * EL;
+#pragma unroll 8
+    for (int v = threadIdx.x; v < ne * EL; v += SPEED_THREADS) sm[v / EL * ES + v % EL] = (float)__ldg(src + v);
+    __syncthreads();
+    float lo = 0.f;
+    if (threadIdx.x < ne) {
+        const float *const m = sm + threadIdx.x * ES;
+        float q[3][N][N], err[3];
+        float lmax[N];   // max over the points of |L_a|, rounded up
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            lmax[a] = 0.f;
+#pragma unroll
+            for (int r = 0; r < N; ++r) lmax[a] = fmaxf(lmax[a], fabsf((float)B.LV[a][r]));
+            lmax[a] *= 1.000001f;
+        }
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+            float t[N][N], sum = 0.f;
+#pragma unroll
+            for (int b = 0; b < N; ++b) {
+                float row = 0.f;
+#pragma unroll
+                for (int r = 0; r < N; ++r) t[b][r] = 0.f;
+#pragma unroll
+                for (int a = 0; a < N; ++a) {
+                    const float x = m[f * NP + b * N + a];
+                    row = fmaf(fabsf(x), lmax[a], row);
+#pragma unroll
+                    for (int r = 0; r < N; ++r) t[b][r] = fmaf((float)B.LV[a][r], x, t[b][r]);
+                }
+                sum = fmaf(row, lmax[b], sum);
+            }
+            err[f] = sum * 0x1p-19f;
+#pragma unroll
+            for (int p = 0; p < N; ++p)
+#pragma unroll
+                for (int r = 0; r < N; ++r) {
+                    float v = 0.f;
+#pragma unroll
+                    for (int b = 0; b < N; ++b) v = fmaf((float)B.LV[b][p], t[b][r], v);
+                    q[f][p][r] = v;
+                }
+        }
+        const float em = 1.5f * fmaxf(err[1], err[2]);
+        float up = 0.f;
+#pragma unroll
+        for (int p = 0; p < N; ++p)
+#pragma unroll
+            for (int r = 0; r < N; ++r) {
+                const float h = href + q[0][p][r], eh = fmaf(fabsf(h) + href, 0x1p-22f, err[0]);
+                const float hl = h - eh, hh = h + eh;
+                const float mom = sqrtf(fmaf(q[1][p][r], q[1][p][r], q[2][p][r] * q[2][p][r]));
+                const float us = ((mom + em) / hl + sqrtf(g * hh)) * 1.00001f;
+                // (a comparison that fails on NaN: the element is left to the FP64 pass)
+                if (!(hl > 0.f) || !(us < 3.0e38f)) up = INFINITY;
+                else {
+                    up = fmaxf(up, us);
+                    lo = fmaxf(lo, (fmaxf(mom - em, 0.f) / hh + sqrtf(g * hl)) * 0.99999f);
+                }
+            }
+        upper[e0 + threadIdx.x] = up;
+    }
+    for (int o = 16; o > 0; o >>= 1) lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    if ((threadIdx.x & 31) == 0 && lo > 0.f) atomicMax(lower, __float_as_uint(lo));   // positive floats order like their bits
+}
+
+// The FP64 pass: each warp looks through 32 elements' bounds and evaluates
+// those that can hold the maximum, one point per lane (several elements at a
+// time at the low degrees).  Positive doubles
+// order like their bit patterns, so an atomic max on the bits is exact and
+// order independent.
+template <typename T, int N>
+__global__ void max_speed_kernel(const T *__restrict__ u, int nel, double href, double g, const float *__restrict__ upper,
+                                 const unsigned *__restrict__ lower, unsigned long long *maxbits, unsigned *status)
 {
     const BasisTab<T> &B = c_basis[N - 1];
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, e0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
+    const float lo = __uint_as_float(*lower);
+    unsigned todo = __ballot_sync(0xffffffffu, e0 + lane < nel && !(upper[min(e0 + lane, nel - 1)] < lo));
     double best = 0.0;
     unsigned st = 0;
-    if (e < nel) {
-        const T *ue = u + (size_t)e * 3 * N * N;
-        for (int q = 0; q < N; ++q)
-            for (int r = 0; r < N; ++r) {
-                double qv[3];
-                for (int f = 0; f < 3; ++f) {
-                    double s = 0.0;
-                    for (int b = 0; b < N; ++b) {
-                        double t = 0.0;
-                        for (int a = 0; a < N; ++a) t += (double)B.LV[a][r] * (double)ue[f * N * N + b * N + a];
-                        s += (double)B.LV[b][q] * t;
-                    }
-                    qv[f] = s;
-                }
-                const double h = href + qv[0];
-                if (!(h > 0.0)) { st |= DG_STATUS_NONPHYSICAL; continue; }
+    constexpr int EPW = 32 / (N * N);   // elements at a time
+    const int grp = min(lane / (N * N), EPW - 1), k = min(lane - grp * N * N, N * N - 1), q = k / N, r = k - q * N;
+    while (todo) {
+        unsigned mine = todo;   // this group's element: the grp-th left
+#pragma unroll
+        for (int i = 0; i < EPW; ++i) {
+            if (i < grp) mine &= mine - 1;
+            todo &= todo - 1;
+        }
+        const bool valid = mine && lane < EPW * N * N;
+        const T *ue = u + (size_t)(e0 + (mine ? __ffs(mine) - 1 : 0)) * 3 * N * N;
+        // lane (b, r) forms the lambda sum of mode row b at point r once, lane
+        // (q, r) collects them over b
+        double qv[3];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+            double t = 0.0, s = 0.0;
+#pragma unroll
+            for (int a = 0; a < N; ++a) t += (double)B.LV[a][r] * (double)ue[f * N * N + q * N + a];
+#pragma unroll
+            for (int b = 0; b < N; ++b) s += (double)B.LV[b][q] * __shfl_sync(0xffffffffu, t, grp * N * N + b * N + r);
+            qv[f] = s;
+        }
+        if (valid) {
+            const double h = href + qv[0];
+            if (!(h > 0.0)) st |= DG_STATUS_NONPHYSICAL;
+            else {
                 const double uu = qv[1] / h, vv = qv[2] / h;
                 best = fmax(best, sqrt(uu * uu + vv * vv) + sqrt(g * h));
             }
+        }
     }
     for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if ((threadIdx.x & 31) == 0 && best > 0.0) atomicMax(maxbits, (unsigned long long)__double_as_longlong(best));
+    if (lane == 0 && best > 0.0) atomicMax(maxbits, (unsigned long long)__double_as_longlong(best));
     if (st) atomicOr(status, st);
 }
 
@@ -1613,19 +1718,24 @@ int dg_launch_mass<DG_REAL>(const DG_REAL *u, const DG_REAL *lo, const double *c
 
 template <>
 int dg_launch_max_speed<DG_REAL>(const DG_REAL *u, int nlon, int nlat, int n, double href, double g,
-                                 unsigned long long *maxbits, unsigned int *status, void *stream)
+                                 unsigned long long *maxbits, float *upper, unsigned int *status, void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int nel = nlon * nlat;
-    const int threads = 128;
-    const int blocks = (nel + threads - 1) / threads;
+    unsigned *const lower = reinterpret_cast<unsigned *>(maxbits + 1);
+    if (cudaMemsetAsync(maxbits, 0, 2 * sizeof(unsigned long long), s) != cudaSuccess) return 1;
+    const int bb = (nel + dgk::SPEED_THREADS - 1) / dgk::SPEED_THREADS, threads = 128, blocks = (nel + threads - 1) / threads;
+#define DG_MS(NN)                                                                                                     \
+    dgk::speed_bound_kernel<DG_REAL, NN><<<bb, dgk::SPEED_THREADS, 0, s>>>(u, nel, (float)href, (float)g, upper, lower); \
+    dgk::max_speed_kernel<DG_REAL, NN><<<blocks, threads, 0, s>>>(u, nel, href, g, upper, lower, maxbits, status)
     switch (n) {
-    case 1: dgk::max_speed_kernel<DG_REAL, 1><<<blocks, threads, 0, s>>>(u, nel, href, g, maxbits, status); break;
-    case 2: dgk::max_speed_kernel<DG_REAL, 2><<<blocks, threads, 0, s>>>(u, nel, href, g, maxbits, status); break;
-    case 3: dgk::max_speed_kernel<DG_REAL, 3><<<blocks, threads, 0, s>>>(u, nel, href, g, maxbits, status); break;
-    case 4: dgk::max_speed_kernel<DG_REAL, 4><<<blocks, threads, 0, s>>>(u, nel, href, g, maxbits, status); break;
-    case 5: dgk::max_speed_kernel<DG_REAL, 5><<<blocks, threads, 0, s>>>(u, nel, href, g, maxbits, status); break;
+    case 1: DG_MS(1); break;
+    case 2: DG_MS(2); break;
+    case 3: DG_MS(3); break;
+    case 4: DG_MS(4); break;
+    case 5: DG_MS(5); break;
     default: return 1;
     }
+#undef DG_MS
     return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
 }
