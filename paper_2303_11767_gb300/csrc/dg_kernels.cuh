@@ -1117,6 +1117,19 @@ int launch_ept_n(const StageArgs<float> &a, cudaStream_t s)
 }
 #endif
 
+#ifndef DG_REAL_IS_F32
+}  // namespace dgk
+#include "dg_stage_f64pt.cuh"
+namespace dgk {
+template <int N>
+int launch_pt_n(const StageArgs<double> &a, cudaStream_t s)
+{
+    const long long warps = ((long long)a.nlon * a.nlat + PtGeo<N>::E - 1) / PtGeo<N>::E;
+    if (launch_pdl(pt_stage_kernel<N>, dim3((unsigned)warps), dim3(32), 0, s, a) != cudaSuccess) return 1;
+    return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
+}
+#endif
+
 constexpr int DG_SMS = 152;   // SMs of a GB300
 
 template <typename T, int N, int W>
@@ -1174,6 +1187,18 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
             if constexpr (N >= 4) return launch_ept_n<N, 16, 8, N == 5 ? 3 : 4>(a, s);
             else return launch_ept_n<N, 32, 4, N == 3 ? 5 : 6>(a, s);
         }
+    }
+#endif
+#ifndef DG_REAL_IS_F32
+    // One lane per Gauss point on small meshes: up to 9 to 14 of its warps per
+    // SM, where both take the same time.  us per stage, tiles / points: degree 1
+    // 20x10 20.7 / 11.8, 120x60 21.2 / 16.3, 180x90 31.5 / 35.2; degree 2 60x30
+    // 28.8 / 14.4, 90x45 28.6 / 26.3, 120x60 38 / 53; degree 3 50x50 36.3 / 23.7,
+    // 90x45 36.4 / 34.3, 120x60 52 / 65; degree 4 50x25 47.5 / 26.0, 72x36 47 /
+    // 55.  (The whole mesh's rows: a band runs the whole mesh's kernel.)
+    if constexpr (N >= 2) {
+        constexpr long long most = N == 2 ? 14500 : N == 3 ? 4100 : N == 4 ? 4250 : 2100;
+        if ((long long)a.nlon * a.nlat_mesh <= most) return launch_pt_n<N>(a, s);
     }
 #endif
     // Tile rows.  FP64 is bound by the FP64 pipe of the busiest SM: tiles per SM

@@ -1,6 +1,8 @@
 """The FP64 stage at every tile height its launch rule takes (8, 4, 2 rows;
-launch_stage_n in csrc/dg_kernels.cuh), on meshes with ragged last tiles, and
-the planar shallow-water problem on the same kernels.  Tolerances as in
+launch_stage_n in csrc/dg_kernels.cuh), on meshes with ragged last tiles, its
+one-lane-per-point kernel (csrc/dg_stage_f64pt.cuh) on the meshes below its line
+(every RK kind, the status bits, bands, the global alpha), and the planar
+shallow-water problem on both.  Tolerances as in
 test_parity_gpu.py (tendencies, 3e-14 of the magnitude bound) and
 test_plane_gpu.py (1e-12)."""
 import numpy as np
@@ -8,7 +10,8 @@ import pytest
 
 import oracle as O
 from paper_2303_11767_gb300 import dgswe
-from test_parity_gpu import assert_within, case, tend_err
+from test_bands_gpu import _run_bands, _whole
+from test_parity_gpu import assert_within, case, state_err, tend_err
 
 pytestmark = pytest.mark.gpu
 
@@ -26,7 +29,7 @@ def tile_rows(nlon, nlat, n):
     return rows
 
 
-MESHES = [(0, 7, 9, 2), (0, 97, 77, 4), (1, 7, 9, 2), (1, 49, 78, 4), (2, 7, 9, 2), (2, 31, 77, 4), (2, 102, 83, 8), (3, 7, 9, 2), (3, 25, 78, 4), (3, 82, 83, 8), (4, 7, 9, 2), (4, 19, 77, 4), (4, 61, 83, 8)]
+MESHES = [(0, 9, 7, 2), (0, 65, 102, 4), (0, 193, 131, 8), (1, 129, 133, 2), (1, 129, 129, 4), (1, 148, 98, 8), (2, 41, 121, 2), (2, 228, 18, 4), (2, 61, 131, 8), (3, 129, 33, 2), (3, 39, 109, 4), (3, 49, 131, 8), (4, 230, 13, 2), (4, 117, 18, 4), (4, 37, 131, 8)]
 
 
 @pytest.mark.parametrize("p,nlon,nlat,rows", MESHES)
@@ -39,9 +42,8 @@ def test_rhs_matches_oracle(p, nlon, nlat, rows):
     assert_within(tend_err(k, o.rhs(u), o.rhs_magnitude(u), what), 3e-14, what)
 
 
-@pytest.mark.parametrize("p,nx,ny,rows", [(3, 50, 50, 4), (1, 33, 53, 2), (3, 49, 66, 4), (4, 79, 66, 8), (2, 5, 1, 2), (4, 1, 3, 2)])
-def test_plane_swe_matches_oracle(p, nx, ny, rows):
-    assert tile_rows(nx, ny, p + 1) == rows
+@pytest.mark.parametrize("p,nx,ny", [(3, 50, 50), (1, 129, 113), (3, 81, 66), (4, 79, 66), (2, 5, 1), (4, 1, 3), (1, 7, 3), (3, 5, 1)])
+def test_plane_swe_matches_oracle(p, nx, ny):
     L = 1.0e6
     with dgswe.Solver.plane_swe(nx, ny, p, L=L) as s:
         lam, th = s.projection_nodes()
@@ -51,3 +53,44 @@ def test_plane_swe_matches_oracle(p, nx, ny, rows):
         k = s.rhs(u)
     o = O.Oracle.plane_swe(nx, ny, p, L, dgswe.GRAVITY, 1.0e-4)
     assert_within(tend_err(k, o.rhs(u), o.rhs_magnitude(u)), 3e-14, f"plane p={p} {nx}x{ny}")
+
+
+POINTS = [(1, 7, 5), (1, 33, 19), (2, 7, 5), (2, 31, 18), (3, 7, 5), (3, 25, 17), (4, 7, 5), (4, 19, 13), (1, 2, 2), (4, 1, 2)]
+
+
+@pytest.mark.parametrize("p,nlon,nlat", POINTS)
+def test_point_stage_rhs_matches_oracle(p, nlon, nlat):
+    o, u = case(nlon, nlat, p, 11)
+    with dgswe.Solver(nlon, nlat, p, precision="fp64") as s:
+        k = s.rhs(u)
+        what = f"rhs p={p} {nlon}x{nlat} fp64, lane per point"
+        assert_within(tend_err(k, o.rhs(u), o.rhs_magnitude(u), what), 3e-14, what)
+        s.set_option(dgswe.OPT_ALPHA_MODE, 1)
+        k = s.rhs(u)
+    o2 = O.Oracle.sphere(nlon, nlat, p, dgswe.EARTH_RADIUS, dgswe.GRAVITY, dgswe.OMEGA)
+    o2.set_alpha_mode(1)
+    assert_within(tend_err(k, o2.rhs(u), o2.rhs_magnitude(u)), 3e-14, what + ", global alpha")
+
+
+@pytest.mark.parametrize("order", [1, 2, 3, 4])
+@pytest.mark.parametrize("p,nlon,nlat", [(1, 33, 19), (2, 31, 18), (3, 25, 17), (4, 19, 13)])
+def test_point_stage_steps_and_bands(p, nlon, nlat, order):
+    torch = pytest.importorskip("torch")
+    o, u = case(nlon, nlat, p, 11)
+    dt = o.max_dt(u, 0.1)
+    whole = _whole(u, nlon, nlat, p, "fp64", 4, dt, order, torch)[0]
+    assert_within(state_err(whole, o.step(u, 4, dt, order)), 1e-12, f"RK{order} p={p}")
+    assert np.array_equal(_run_bands(u, nlon, nlat, p, "fp64", 3, 4, dt, order, torch)[0], whole)
+
+
+@pytest.mark.parametrize("j,i", [(0, 0), (12, 18), (6, 9)])
+@pytest.mark.parametrize("value,status", [(np.nan, dgswe.DG_ENONFINITE), (-3.0e4, dgswe.DG_ENONPHYSICAL), (np.inf, dgswe.DG_ENONFINITE)])
+def test_point_stage_reports_bad_states(j, i, value, status):
+    _, u = case(19, 13, 4, 11)
+    bad = u.copy()
+    bad[j, i, 0, 0] = value
+    with dgswe.Solver(19, 13, 4, precision="fp64") as s:
+        with pytest.raises(dgswe.DGError) as e:
+            s.rhs(bad)
+        assert e.value.status == status
+        s.rhs(u)
