@@ -1233,12 +1233,17 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
 // One persistent launch per RK stage for a batch of meshes of different sizes
 // and degrees: every CTA walks the work list (member, tile column, tile row)
 // and runs the tile with the member's degree.  Items are ordered by cost,
-// largest first, so the round-robin walk balances the CTAs.
+// largest first, and every other round is walked backwards, so the CTAs with
+// the longest first tiles get the shortest second ones (12 members of 20 to 60
+// rows, two CTAs per SM: 22.2 -> 20.8 us per stage).
 template <typename T, int W>
 __global__ void __launch_bounds__(32 * W, 24 / W) ensemble_kernel(const EnsArgs<T> E)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    for (int it = blockIdx.x; it < E.nitems; it += gridDim.x) {
+    pdl_wait();
+    for (int r = 0, first = 0; first < E.nitems; ++r, first += gridDim.x) {
+        const int it = first + (int)(r & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+        if (it >= E.nitems) continue;   // (the whole block)
         const EnsItem item = E.items[it];
         const EnsMember<T> m = E.members[item.member];
         StageArgs<T> A;
@@ -1309,7 +1314,7 @@ int launch_ensemble_w(int grid, const EnsArgs<T> &a, cudaStream_t s)
             return 1;
         attr_set.fetch_or(1ull << dev, std::memory_order_release);   // setting it twice is harmless
     }
-    ensemble_kernel<T, W><<<grid, 32 * W, smem, s>>>(a);
+    if (launch_pdl(ensemble_kernel<T, W>, dim3(grid), dim3(32 * W), smem, s, a) != cudaSuccess) return 1;
     return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
 }
 
