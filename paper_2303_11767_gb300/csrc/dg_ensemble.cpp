@@ -260,6 +260,9 @@ dg_status dg_ensemble_create(int members, const int *nlon, const int *nlat, cons
                     d.cosn[a] = (float)s.cosn[a];
                     d.sinn[a] = (float)s.sinn[a];
                     d.rho[a] = (float)s.rho[a];
+                    d.cGc[a] = (float)(2.0 / (radius * e->tabs[m].dth) * s.cosn[a]);
+                    d.sR[a] = (float)(s.sinn[a] / radius);
+                    d.fc[a] = (float)(2.0 * omega * s.sinn[a] * s.cosn[a]);
                     d.CSE[a] = (float)s.CSE[a];
                     d.CSW[a] = (float)s.CSW[a];
                     for (int b = 0; b < DG_MAXN; ++b) {

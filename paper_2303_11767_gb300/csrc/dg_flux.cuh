@@ -135,9 +135,10 @@ __device__ __forceinline__ void rusanov_out(const T *L, const T *R, const T *fl,
 #pragma unroll
         for (int f = 0; f < 3; ++f) out[f] = hc * fma(-a, R[f] - L[f], __dadd_rn(fl[f], fr[f]));
     } else {
-        const T ha = T(0.5) * (aglob > T(0) ? aglob : fmax(al, ar));   // global mode: the stage's largest |u| + c
+        const T a = aglob > T(0) ? aglob : fmax(al, ar);   // global mode: the stage's largest |u| + c
+        const T hc = T(0.5) * c;
 #pragma unroll
-        for (int f = 0; f < 3; ++f) out[f] = c * fma(-ha, R[f] - L[f], T(0.5) * (fl[f] + fr[f]));
+        for (int f = 0; f < 3; ++f) out[f] = hc * fma(-a, R[f] - L[f], fl[f] + fr[f]);
     }
 }
 

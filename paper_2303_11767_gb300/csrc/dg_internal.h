@@ -30,7 +30,7 @@ struct BasisTab {
 //   rho: hv tendency of the (a = 0, b) modes produced by a unit constant
 //        pressure flux (the rest state with g h^2 / 2 = 1), n-point rules
 //   cGc, sR, fc: cG cos, sin / R and 2 Omega sin cos at the Gauss points, the
-//        row constants of the FP64 stage's pointwise phase (filled at upload)
+//        row constants of the stage's pointwise phase (filled at upload)
 template <typename T>
 struct RowTab {
     T cosn[DG_MAXN];

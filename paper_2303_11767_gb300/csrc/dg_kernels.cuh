@@ -817,6 +817,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
             GsS[f] = ef[(own * 2 + 1) * 3 * N + f * N + k];
             GsN[f] = (valid && (j < A.nlat - 1 || A.halo_n)) ? ef[((own + TW) * 2 + 1) * 3 * N + f * N + k] : T(0);
         }
+        const T hg = T(0.5) * gg, gH = gg * href;
         T X1[3][N], X2[3][N];
 #pragma unroll
         for (int f = 0; f < 3; ++f)
@@ -833,21 +834,13 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
             const T rh = rcp(h);
             const T u = hu * rh, v = hv * rh;
             T F0, F1, F2, G0, G1, G2, S1, S2;
-            if constexpr (sizeof(T) == 8) {   // the row's constants folded: 20 operations per point instead of 35
-                const T P = pressure(hp, href, gg);
+            {   // the row's constants folded: 20 operations per point instead of 35
+                const T P = hp * fma(hg, hp, gH);
                 const T cGc = __ldg(&RT->cGc[q]), sR = __ldg(&RT->sR[q]);
                 F0 = A.cF * hu, F1 = fma(F0, u, A.cF * P), F2 = F0 * v;
                 G0 = cGc * hv, G1 = G0 * u, G2 = fma(G0, v, cGc * P);
                 const T K = fma(u, sR, __ldg(&RT->fc[q]));
                 S1 = K * hv, S2 = fma(-K, hu, -(P * sR));
-            } else {
-                const T P = hp * gg * (href + T(0.5) * hp);
-                const T c = __ldg(&RT->cosn[q]), s = __ldg(&RT->sinn[q]);
-                F0 = A.cF * hu, F1 = A.cF * fma(hu, u, P), F2 = A.cF * (hu * v);
-                const T cGc = A.cG * c;
-                G0 = cGc * hv, G1 = cGc * (hv * u), G2 = cGc * fma(hv, v, P);
-                const T K = s * fma(A.twoOmega, c, u * A.invR);
-                S1 = K * hv, S2 = -(P * s * A.invR) - K * hu;
             }
             constexpr int PL = pair_len<T, N>();
             if constexpr (PL > 0) {
@@ -913,9 +906,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
                 ye = fma(Qk[q], efE[f * N + q], ye);
                 yw = fma(Qk[q], efW[f * N + q], yw);
             }
+            // E / W lift: -(L_a(1) ye - L_a(-1) yw), L_a(-1) = (-1)^a L_a(1)
+            const T ed = yw - ye, es = -(yw + ye);
             if constexpr (sizeof(T) == 8) {
-                // even-odd split of w L_a and w L_a' over the points q, N-1-q,
-                // and of the edge values L_a(+-1)
+                // even-odd split of w L_a and w L_a' over the points q, N-1-q
                 T p1[(N + 1) / 2], m1[(N + 1) / 2], p2[(N + 1) / 2], m2[(N + 1) / 2];
 #pragma unroll
                 for (int q = 0; q < N / 2; ++q) {
@@ -925,7 +919,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
                     m2[q] = y2[q] - y2[N - 1 - q];
                 }
                 if constexpr (N % 2) p1[N / 2] = y1[N / 2], p2[N / 2] = y2[N / 2];
-                const T ed = yw - ye, es = -(yw + ye);
 #pragma unroll
                 for (int a = 0; a < N; ++a) {
                     T s = B.SE[a] * (a % 2 ? es : ed);
@@ -948,8 +941,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
                     for (int q = 0; q < N; ++q)
                         s = __ffma2_rn(f2(B.WLD[a][q], B.WLD[a + 1][q]), bc2(y1[q]),
                                        __ffma2_rn(f2(B.WLV[a][q], B.WLV[a + 1][q]), bc2(y2[q]), s));
-                    kk[f][a] = s.x - (B.SE[a] * ye - B.SW[a] * yw);
-                    kk[f][a + 1] = s.y - (B.SE[a + 1] * ye - B.SW[a + 1] * yw);
+                    s = __ffma2_rn(f2(B.SE[a], B.SE[a + 1]), f2(ed, es), s);
+                    kk[f][a] = s.x;
+                    kk[f][a + 1] = s.y;
                 }
             }
 #pragma unroll
@@ -957,7 +951,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
                 T s = T(0);
 #pragma unroll
                 for (int q = 0; q < N; ++q) s = fma(B.WLD[a][q], y1[q], fma(B.WLV[a][q], y2[q], s));
-                kk[f][a] = s - (B.SE[a] * ye - B.SW[a] * yw);
+                kk[f][a] = fma(B.SE[a], a % 2 ? es : ed, s);
             }
         }
         kk[2][0] = fma(A.P0, rhok, kk[2][0]);
@@ -1087,6 +1081,8 @@ constexpr size_t stage_smem_bytes()
     return SmemMap<T, N, W>::BYTES;
 }
 
+constexpr int DG_SMS = 152;   // SMs of a GB300
+
 #ifdef DG_REAL_IS_F32
 }  // namespace dgk
 #include "dg_stage_ept.cuh"
@@ -1130,7 +1126,6 @@ int launch_pt_n(const StageArgs<double> &a, cudaStream_t s)
 }
 #endif
 
-constexpr int DG_SMS = 152;   // SMs of a GB300
 
 template <typename T, int N, int W>
 int launch_stage_w(const StageArgs<T> &a, cudaStream_t s)
@@ -1175,15 +1170,24 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // One thread per element where the mesh has enough elements for it; else
     // N lanes per element, whose tiles have the shorter chain (one tile takes
     // 8 instead of 13 us at degree 4).  The line lies where both take the same
-    // time; us per stage, lanes / threads: degree 4 180x90 13.9 / 13.2, 360x180
-    // 40.5 / 34.8, 1440x720 586 / 380; degree 3 180x90 5.85 / 8.5, 360x180 16.5
-    // / 14.5, 1440x720 235 / 204; degree 2 120x60 5.1 / 6.1, 241x121 8.6 / 7.2,
-    // 720x360 53.9 / 29.7; degree 1 120x60 3.4 / 4.0, 720x360 18.7 / 14.7.
+    // time; us per stage, lanes / threads: degree 4 180x90 13.9 / 13.1, 360x180
+    // 40.5 / 30.1, 1440x720 586 / 373; degree 3 180x90 5.85 / 8.5, 360x180 16.5
+    // / 14.4, 1440x720 235 / 202; degree 2 120x60 5.0 / 6.1, 241x121 8.6 / 6.9,
+    // 720x360 53.9 / 29.2; degree 1 120x60 3.4 / 4.0, 720x360 18.7 / 14.7.
     // It counts the whole mesh's rows, so that a latitude band of a mesh runs
     // the kernel of the whole mesh and gets its bits.
     if constexpr (N >= 2) {
         constexpr long long least = N == 5 ? 14000 : N == 4 ? 40000 : 18000;
         if ((long long)a.nlon * a.nlat_mesh >= least) {
+            if constexpr (N == 5) {
+                // three tiles run on an SM at a time; where 16 x 8 tiles need a
+                // little more than one round of them, the second round runs nearly
+                // alone, and tiles of 32 x 4, whose last column is cheap, end
+                // sooner (us per stage, 16 x 8 / 32 x 4: 330x165 21.9 / 29.4,
+                // 360x180 33.1 / 30.1, 380x190 34.1 / 30.9, 400x200 35.4 / 41.6)
+                const long long t = ((a.nlon + 15) / 16) * ((a.nlat + 7) / 8);
+                if (t > 3 * DG_SMS && t <= 4 * DG_SMS) return launch_ept_n<5, 32, 4, 3>(a, s);
+            }
             if constexpr (N >= 4) return launch_ept_n<N, 16, 8, N == 5 ? 3 : 4>(a, s);
             else return launch_ept_n<N, 32, 4, N == 3 ? 5 : 6>(a, s);
         }
@@ -1288,6 +1292,7 @@ __global__ void __launch_bounds__(32 * W, 24 / W) ensemble_kernel(const EnsArgs<
         }
         __syncthreads();   // the next item reuses the shared memory
     }
+    pdl_launch_dependents();
 }
 
 template <typename T, int W>

@@ -456,13 +456,14 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
         ept_lift<float, N>(B, RT, fs, KN, N * KN, TX, k0);
         ept_lift<float2, N>(B, RT, fs + N * KN, KN, N * KN, TX, k1);
     }
+    const float hg = 0.5f * gg, gH = gg * href;
 #pragma unroll 1
     for (int be = 0; be < N; ++be) {
         float x0[N];
         float2 x1[N];
         ept_get_row<float, N>(me + be * N, NP, x0);
         ept_get_row<float2, N>(me + NP + be * N, NP, x1);
-        const float c = __ldg(&RT->cosn[be]), s = __ldg(&RT->sinn[be]), cGc = A.cG * c;
+        const float cGc = __ldg(&RT->cGc[be]), sR = __ldg(&RT->sR[be]), fc = __ldg(&RT->fc[be]);
         float Y10[N], Y20[N];    // coefficients of QT and PT: h
         float2 Y11[N], Y21[N];   // (hu, hv)
         {
@@ -485,12 +486,12 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
             hmin = fmin(hmin, h);
             const float rh = rcp(h);
             const float u = hu * rh, v = hv * rh;
-            const float P = hp * gg * fma(0.5f, hp, href);
+            const float P = hp * fma(hg, hp, gH);
             const float F0 = A.cF * hu, G0 = cGc * hv;
-            const float2 F1 = __fmul2_rn(bc2(A.cF), f2(fma(hu, u, P), hu * v));
-            const float2 G1 = __fmul2_rn(bc2(cGc), f2(hv * u, fma(hv, v, P)));
-            const float K = s * fma(A.twoOmega, c, u * A.invR);
-            const float2 S1 = f2(K * hv, fma(-K, hu, -(P * s * A.invR)));
+            const float2 F1 = f2(fma(F0, u, A.cF * P), F0 * v);
+            const float2 G1 = f2(G0 * u, fma(G0, v, cGc * P));
+            const float K = fma(u, sR, fc);
+            const float2 S1 = f2(K * hv, fma(-K, hu, -(P * sR)));
 #pragma unroll
             for (int a = 0; a < N; ++a) {
                 const float wd = B.WLD[a][al], wl = B.WLV[a][al];
@@ -550,7 +551,7 @@ __device__ __forceinline__ void ept_tile(const StageArgs<float> &A, int bx, int 
                 chk = nf_acc(pb.x, nf_acc(pb.y, chk));
             }
         };
-        constexpr int EB = FIN == 0 ? RBL : (RBL + 1) / 2;
+        constexpr int EB = N == 5 ? (RBL + 3) / 4 : FIN == 0 ? RBL : (RBL + 1) / 2;   // (measured: degree 4 373 against 377 us, degree 3 202 against 208)
 #pragma unroll 1
         for (int rr = 0; rr < RPW; ++rr) {
             const int r = warp * RPW + rr;
