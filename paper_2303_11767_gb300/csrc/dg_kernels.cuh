@@ -1170,14 +1170,16 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // One thread per element where the mesh has enough elements for it; else
     // N lanes per element, whose tiles have the shorter chain (one tile takes
     // 8 instead of 13 us at degree 4).  The line lies where both take the same
-    // time; us per stage, lanes / threads: degree 4 180x90 13.9 / 13.1, 360x180
-    // 40.5 / 30.1, 1440x720 586 / 373; degree 3 180x90 5.85 / 8.5, 360x180 16.5
-    // / 14.4, 1440x720 235 / 202; degree 2 120x60 5.0 / 6.1, 241x121 8.6 / 6.9,
-    // 720x360 53.9 / 29.2; degree 1 120x60 3.4 / 4.0, 720x360 18.7 / 14.7.
+    // time; us per stage, lanes / threads: degree 4 160x80 10.9 / 13.1, 200x100
+    // 14.2 / 14.5, 240x120 19.8 / 14.6, 360x180 40.5 / 30.1, 1440x720 586 / 373;
+    // degree 3 220x110 7.3 / 9.4, 260x130 10.2 / 9.6, 360x180 16.5 / 14.4,
+    // 1440x720 235 / 202; degree 2 180x90 6.6 / 6.3, 220x110 8.0 / 6.7, 720x360
+    // 53.9 / 29.2; degree 1 300x150 4.9 / 5.2, 360x180 7.1 / 5.8, 720x360 18.7 /
+    // 15.2.
     // It counts the whole mesh's rows, so that a latitude band of a mesh runs
     // the kernel of the whole mesh and gets its bits.
     if constexpr (N >= 2) {
-        constexpr long long least = N == 5 ? 14000 : N == 4 ? 40000 : 18000;
+        constexpr long long least = N == 5 ? 21000 : N == 4 ? 32000 : N == 3 ? 18000 : 50000;
         if ((long long)a.nlon * a.nlat_mesh >= least) {
             if constexpr (N == 5) {
                 // three tiles run on an SM at a time; where 16 x 8 tiles need a

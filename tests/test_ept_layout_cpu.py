@@ -7,14 +7,14 @@ output blocks of all tiles together write every own value exactly once."""
 import numpy as np
 import pytest
 
-GEOMETRY = {2: (32, 4), 3: (32, 4), 4: (16, 8), 5: (16, 8)}   # N -> tile columns, rows
+GEOMETRY = [(2, 32, 4), (3, 32, 4), (4, 16, 8), (5, 16, 8), (5, 32, 4)]   # N, tile columns, rows
 MESHES = [(1, 3), (2, 9), (4, 2), (15, 19), (16, 8), (33, 5), (35, 19), (67, 9), (64, 13)]
 
 
 class Geo:
-    def __init__(self, N):
+    def __init__(self, geometry):
+        N, self.TX, self.TY = geometry
         self.N, self.EL = N, 3 * N * N
-        self.TX, self.TY = GEOMETRY[N]
         self.VEC = (N * N) % 4 == 0
         EL = self.EL
         self.ES = (EL if (EL // 4) % 2 else EL + 4) if self.VEC else EL
@@ -35,10 +35,10 @@ class Geo:
         return (c // (self.EL // 4)) * self.ES + c % (self.EL // 4) * 4 if self.VEC else 4 * c
 
 
-@pytest.mark.parametrize("N", sorted(GEOMETRY))
-def test_shared_memory_fits(N):
-    g = Geo(N)
-    ctas = {2: 6, 3: 5, 4: 4, 5: 3}[N]
+@pytest.mark.parametrize("geometry", GEOMETRY)
+def test_shared_memory_fits(geometry):
+    g = Geo(geometry)
+    ctas = {(2, 32): 6, (3, 32): 5, (4, 16): 4, (5, 16): 3, (5, 32): 2}[geometry[:2]]
     assert g.U % 4 == 0 and g.ROW % 4 == 0 and g.SLOT % 4 == 0
     assert ctas * (4 * g.LEN + 1024) <= 228 * 1024
     # the lanes of a warp read word m of 32 elements (or 16-byte block m of 8)
@@ -51,9 +51,9 @@ def test_shared_memory_fits(N):
 
 @pytest.mark.parametrize("gs,gn", [(0, 0), (1, 0), (1, 1)])
 @pytest.mark.parametrize("nlon,nlat", MESHES)
-@pytest.mark.parametrize("N", sorted(GEOMETRY))
-def test_tiles(N, nlon, nlat, gs, gn):
-    g = Geo(N)
+@pytest.mark.parametrize("geometry", GEOMETRY)
+def test_tiles(geometry, nlon, nlat, gs, gn):
+    g = Geo(geometry)
     EL, TX, TY = g.EL, g.TX, g.TY
     row = nlon * EL
     base = gs * row                                        # own row 0; the array starts 16-byte aligned
