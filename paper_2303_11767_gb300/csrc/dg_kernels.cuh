@@ -1209,27 +1209,38 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
 #endif
     // Tile rows.  FP64 is bound by the FP64 pipe of the busiest SM: tiles per SM
     // x rows x the cost of a row in a tile of that height (a short tile has more
-    // ring traces and evaluates more of its boundary edges twice).  Measured at
-    // 8, 4, 2, 1 rows (us per stage): 20x10 degree 1 36.4 23.8 23.3 26.8 (4 tiles
-    // of 8 rows ran on 4 SMs); 50x50 degree 3 69 44 44 48; 120x60 degree 2 52.6
-    // 53.3 46.2 50.3; 180x90 degree 3 138 143 154 180; 360x180 degree 4 906 821
-    // 901 1118: a row costs 1, 1.02, 1.2 and 1.5, and one-row tiles never win.
-    // FP32 takes 8 rows (90x45 degree 3 4.5 4.7 5.2 5.9; 180x90 5.9 6.2 7.6 11.9).
-    int w = DG_WARPS;
-    if (sizeof(T) == 8) {
+    // ring traces and evaluates more of its boundary edges twice).  A quarter of
+    // the SM with one warp more than the others counts 3.5 rows per warp: a
+    // single tile of 5 rows takes as long as one of 7.  Measured at 8, 7, 5, 4,
+    // 2 rows (us per stage; more heights to choose from, fewer SMs that wait):
+    // 180x90 degree 3 108 102 112 115 132; 120x60 degree 3 53.7 50.6 71.2 58.1
+    // 52.1; 360x180 degree 4 692 693 651 648 725; 90x45 degree 4 71.6 64.7 70.8
+    // 74.7 65.3; 240x120 degree 2 124 113 104 127 141, degree 1 60.9 50.6 62.0
+    // 45.4 65.4; 300x150 degree 0 39.9 32.4 25.3 29.2 29.0.  Heights 6 and 3 win
+    // nowhere by more than 3 % (360x180 degree 3 362 against 370), one row never.
+    // FP32 takes 8 rows (90x45 degree 3 4.5, 4 rows 4.7; 180x90 5.9 6.2).
+    if constexpr (sizeof(T) == 8) {
+        constexpr int rows[] = {8, 7, 5, 4, 2};
+        constexpr double cost[] = {1.0, 1.02, 1.03, 1.04, 1.2};
+        int w = DG_WARPS;
         double best = 0;
-        for (int c = DG_WARPS; c >= 2; c /= 2) {
-            const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((a.nlat + c - 1) / c);
-            const double work = (double)((tiles + DG_SMS - 1) / DG_SMS) * c * (c == 8 ? 1.0 : c == 4 ? 1.02 : 1.2);
-            if (c == DG_WARPS || work < best) {
+        for (int c = 0; c < 5; ++c) {
+            const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((a.nlat + rows[c] - 1) / rows[c]);
+            const long long per_sm = (tiles + DG_SMS - 1) / DG_SMS * rows[c];
+            const double quarter = 3.5 * (double)((per_sm + 3) / 4);
+            const double work = cost[c] * (quarter > (double)per_sm ? quarter : (double)per_sm);
+            if (c == 0 || work < best) {
                 best = work;
-                w = c;
+                w = rows[c];
             }
         }
-    }
-    if constexpr (sizeof(T) == 8) {
-        if (w == 2) return launch_stage_w<T, N, 2>(a, s);
-        if (w == 4) return launch_stage_w<T, N, 4>(a, s);
+        switch (w) {
+        case 2: return launch_stage_w<T, N, 2>(a, s);
+        case 4: return launch_stage_w<T, N, 4>(a, s);
+        case 5: return launch_stage_w<T, N, 5>(a, s);
+        case 7: return launch_stage_w<T, N, 7>(a, s);
+        default: break;
+        }
     }
     return launch_stage_w<T, N, DG_WARPS>(a, s);
 }

@@ -1,4 +1,4 @@
-"""The FP64 stage at every tile height its launch rule takes (8, 4, 2 rows;
+"""The FP64 stage at every tile height its launch rule takes (8, 7, 5, 4, 2 rows;
 launch_stage_n in csrc/dg_kernels.cuh), on meshes with ragged last tiles, its
 one-lane-per-point kernel (csrc/dg_stage_f64pt.cuh) on the meshes below its line
 (every RK kind, the status bits, bands, the global alpha), and the planar
@@ -21,15 +21,16 @@ SMS = 152
 def tile_rows(nlon, nlat, n):
     """The launch rule."""
     rows, best = 8, None
-    for c, cost in ((8, 1.0), (4, 1.02), (2, 1.2)):
+    for c, cost in ((8, 1.0), (7, 1.02), (5, 1.03), (4, 1.04), (2, 1.2)):
         tiles = -(-nlon // (32 // n)) * -(-nlat // c)
-        work = -(-tiles // SMS) * c * cost
+        per_sm = -(-tiles // SMS) * c
+        work = cost * max(per_sm, 3.5 * (-(-per_sm // 4)))
         if best is None or work < best:
             rows, best = c, work
     return rows
 
 
-MESHES = [(0, 9, 7, 2), (0, 65, 102, 4), (0, 193, 131, 8), (1, 129, 133, 2), (1, 129, 129, 4), (1, 148, 98, 8), (2, 41, 121, 2), (2, 228, 18, 4), (2, 61, 131, 8), (3, 129, 33, 2), (3, 39, 109, 4), (3, 49, 131, 8), (4, 230, 13, 2), (4, 117, 18, 4), (4, 37, 131, 8)]
+MESHES = [(0, 122, 34, 4), (0, 190, 122, 7), (0, 241, 139, 8), (0, 194, 85, 2), (0, 259, 137, 5), (1, 231, 79, 8), (1, 148, 137, 5), (1, 231, 103, 4), (1, 156, 100, 7), (1, 131, 133, 2), (2, 55, 87, 4), (2, 199, 40, 7), (2, 131, 89, 5), (2, 107, 100, 8), (2, 216, 25, 2), (3, 52, 138, 7), (3, 169, 67, 4), (3, 189, 92, 5), (3, 147, 123, 8), (3, 162, 113, 2), (4, 149, 59, 5), (4, 81, 58, 7), (4, 203, 29, 8), (4, 125, 113, 2), (4, 89, 25, 4)]
 
 
 @pytest.mark.parametrize("p,nlon,nlat,rows", MESHES)
@@ -94,3 +95,13 @@ def test_point_stage_reports_bad_states(j, i, value, status):
             s.rhs(bad)
         assert e.value.status == status
         s.rhs(u)
+
+
+@pytest.mark.parametrize("p,nlon,nlat,rows", [(1, 156, 100, 7), (2, 131, 89, 5), (3, 52, 138, 7)])
+def test_tile_rows_bands_get_the_whole_mesh_bits(p, nlon, nlat, rows):
+    torch = pytest.importorskip("torch")
+    assert tile_rows(nlon, nlat, p + 1) == rows
+    o, u = case(nlon, nlat, p, 11)
+    dt = o.max_dt(u, 0.1)
+    whole = _whole(u, nlon, nlat, p, "fp64", 2, dt, 3, torch)[0]
+    assert np.array_equal(_run_bands(u, nlon, nlat, p, "fp64", 3, 2, dt, 3, torch)[0], whole)
