@@ -90,7 +90,7 @@ typedef enum {
                                     default 16 */
     DG_OPT_TILE_ROWS = 7,        /* ensemble only: latitude rows per CTA tile, 4 or 8
                                     (default 8; dg_ensemble_autotune picks it) */
-    DG_OPT_BLOCKS_PER_SM = 8,    /* ensemble only: persistent CTAs per SM, 1..8 (default 2) */
+    DG_OPT_BLOCKS_PER_SM = 8,    /* ensemble only: persistent CTAs per SM and degree, 1..8 (default 2) */
     DG_OPT_WELL_BALANCED = 9     /* 0 (default) / 1: remove from every tendency that of the
                                     fluid at rest at the reference depth (the mean depth of the
                                     state at dg_set_state), i.e. the quadrature residual of its
@@ -334,7 +334,7 @@ dg_status dg_restrict_from(dg_handle coarse, dg_handle fine);
  * Batched ensemble: many independent meshes of uneven sizes and degrees (the
  * decoupled copies of the 2-D problem of the paper's vertical-levels
  * experiment, Sec. 5.2.2), advanced together in FP32 by one persistent
- * launch per SSP-RK3 stage (Table "Butcher") inside a captured CUDA graph.
+ * launch per SSP-RK3 stage (Table "Butcher") and degree inside a captured CUDA graph.
  * Each member has its own state (same layout as above), its own time step
  * and its own reference depth; members never interact.
  * ------------------------------------------------------------------------ */
@@ -366,7 +366,7 @@ dg_status dg_ensemble_max_dt(dg_ensemble e, int member, double cfl, double *dt);
  * (saved and restored), keeps the fastest and returns it, with the time of
  * one step in ms. */
 dg_status dg_ensemble_autotune(dg_ensemble e, int trials, int *tile_rows, int *blocks_per_sm, double *best_ms);
-/* Persistent stage launches issued so far (one per RK stage). */
+/* RK stages launched so far (of all members; one per RK stage). */
 long long dg_ensemble_stage_launches(dg_ensemble e);
 
 /* The paper has no counterpart to this entry point.

@@ -1,7 +1,7 @@
 // dg_ensemble.cpp -- batched ensemble of independent meshes (uneven sizes and
-// degrees) advanced together: one persistent FP32 launch per SSP-RK stage
-// over all members, captured in a CUDA graph, with a tile-shape / grid-size
-// autotuner.  The members are the decoupled copies of the 2-D problem of the
+// degrees) advanced together: one persistent FP32 launch per SSP-RK stage and
+// degree over all its members, each degree a chain of launches on a stream of
+// its own, captured in a CUDA graph, with a tile-shape / grid-size autotuner.  The members are the decoupled copies of the 2-D problem of the
 // paper's vertical-levels experiment (Sec. 5.2.2), here each with its own
 // mesh, degree and initial field.
 #include <cuda_runtime.h>
@@ -55,7 +55,13 @@ struct dg_ens {
     std::vector<EnsMember<float>> hm;
     EnsMember<float> *dm = nullptr;
     EnsItem *items[2] = {nullptr, nullptr};   // work lists for the two tile heights
-    int nitems[2] = {0, 0};
+    // part of the work list per degree present, highest degree first
+    struct Part {
+        int n, first[2], count[2];
+    };
+    std::vector<Part> parts;
+    cudaStream_t side[DG_MAXN - 1] = {};      // streams of the degrees after the first
+    cudaEvent_t fork = nullptr, join[DG_MAXN - 1] = {};
     double *c0 = nullptr, *partials = nullptr, *d_result = nullptr;
     std::vector<size_t> c0_off;
     int nblocks = 0;
@@ -107,7 +113,7 @@ struct EPlan {
 // SSP-RK3 (Table "Butcher") in increment form, as in the single-mesh solver
 const EPlan kPlan[3] = {{-1, 0, 0, 0, 1}, {0, 1, 0, 0.25, 0.25}, {1, -1, 1, 2.0 / 3.0, 2.0 / 3.0}};
 
-dg_status launch_step(dg_ens *e, int cur)
+dg_status launch_step(dg_ens *e, const dg_ens::Part &part, cudaStream_t stream, int cur)
 {
     const int ti = tile_index(e->tile_rows);
     for (int s = 0; s < 3; ++s) {
@@ -123,20 +129,40 @@ dg_status launch_step(dg_ens *e, int cur)
         }
         a.rows = e->rows;
         a.members = e->dm;
-        a.items = e->items[ti];
-        a.nitems = e->nitems[ti];
+        a.items = e->items[ti] + part.first[ti];
+        a.nitems = part.count[ti];
         a.status = e->d_status;
         a.g = (float)e->g;
         a.invR = (float)(1.0 / e->R);
         a.twoOmega = (float)(2.0 * e->omega);
         a.ci = (float)kPlan[s].ci;
         a.cc = (float)kPlan[s].cc;
-        const int grid = std::max(1, std::min(e->nitems[ti], e->sms * e->bps));
-        if (dg_launch_ensemble_stage<float>(e->tile_rows, grid, a, e->stream))
+        const int grid = std::max(1, std::min(part.count[ti], e->sms * e->bps));
+        if (dg_launch_ensemble_stage<float>(e->tile_rows, part.n, grid, a, stream))
             return efail(DG_ECUDA, "ensemble stage launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-        e->launches++;
     }
     return DG_OK;
+}
+
+// k steps from buffer `cur`: every degree's chain of 3 k launches, the first on
+// the ensemble's stream and the others beside it between a fork and a join.
+// The chains touch disjoint parts of the state arrays.
+dg_status launch_steps(dg_ens *e, int k, int cur)
+{
+    dg_status st = DG_OK;
+    const size_t others = e->parts.size() - 1;
+    size_t forked = 0;
+    if (others && cudaEventRecord(e->fork, e->stream) != cudaSuccess) return efail(DG_ECUDA, "event record failed");
+    for (; forked < others && !st; ++forked)
+        if (cudaStreamWaitEvent(e->side[forked], e->fork, 0) != cudaSuccess) st = efail(DG_ECUDA, "stream wait failed");
+    for (int i = 0; i < k && !st; ++i)
+        for (size_t c = 0; c <= others && !st; ++c)
+            st = launch_step(e, e->parts[c], c ? e->side[c - 1] : e->stream, cur ^ (i & 1));
+    for (size_t c = 0; c < forked; ++c)   // also after a failure: a capture must end joined
+        if ((cudaEventRecord(e->join[c], e->side[c]) != cudaSuccess ||
+             cudaStreamWaitEvent(e->stream, e->join[c], 0) != cudaSuccess) && !st)
+            st = efail(DG_ECUDA, "stream join failed");
+    return st;
 }
 
 dg_status build_items(dg_ens *e)
@@ -148,15 +174,21 @@ dg_status build_items(dg_ens *e)
             const int n = e->deg[m] + 1, G = dg_ensemble_tile_width(n);
             const int tx = (e->nlon[m] + G - 1) / G, ty = (e->nlat[m] + W - 1) / W;
             for (int y = 0; y < ty; ++y)
-                for (int x = 0; x < tx; ++x) it.push_back({m, x, y, n * n * n * 16});   // cost ~ n^3 per element
+                for (int x = 0; x < tx; ++x) it.push_back({m, x, y, n});
         }
-        // largest cost first, then member and position: CTAs that walk the list
-        // round-robin end up with nearly equal work
-        std::stable_sort(it.begin(), it.end(), [](const EnsItem &a, const EnsItem &b) { return a.cost > b.cost; });
+        // by degree, then member and position
+        std::stable_sort(it.begin(), it.end(), [](const EnsItem &a, const EnsItem &b) { return a.n > b.n; });
+        for (size_t i = 0, p = 0; i < it.size(); ++p) {
+            size_t last = i;
+            while (last < it.size() && it[last].n == it[i].n) ++last;
+            if (ti == 0) e->parts.push_back({it[i].n, {0, 0}, {0, 0}});
+            e->parts[p].first[ti] = (int)i;
+            e->parts[p].count[ti] = (int)(last - i);
+            i = last;
+        }
         if (cudaMalloc(&e->items[ti], sizeof(EnsItem) * it.size()) != cudaSuccess)
             return efail(DG_ENOMEM, "cudaMalloc of the work list failed");
         ECUDA(cudaMemcpy(e->items[ti], it.data(), sizeof(EnsItem) * it.size(), cudaMemcpyHostToDevice));
-        e->nitems[ti] = (int)it.size();
     }
     return DG_OK;
 }
@@ -293,6 +325,12 @@ dg_status dg_ensemble_create(int members, const int *nlon, const int *nlat, cons
             ETRY(efail(DG_ECUDA, "table upload failed"));
     }
     ETRY(build_items(e));
+    if (cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming) != cudaSuccess)
+        ETRY(efail(DG_ECUDA, "event creation failed"));
+    for (size_t c = 0; c + 1 < e->parts.size(); ++c)
+        if (cudaStreamCreateWithFlags(&e->side[c], cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&e->join[c], cudaEventDisableTiming) != cudaSuccess)
+            ETRY(efail(DG_ECUDA, "stream creation failed"));
     size_t max_nel = *std::max_element(e->nel.begin(), e->nel.end());
     e->nblocks = dg_mass_blocks(max_nel);
     if (cudaMalloc(&e->partials, 2 * sizeof(double) * e->nblocks) != cudaSuccess ||
@@ -324,6 +362,11 @@ dg_status dg_ensemble_destroy(dg_ensemble e)
     cudaFree(e->d_result);
     cudaFree(e->d_status);
     cudaFree(e->d_maxbits);
+    for (cudaStream_t s : e->side)
+        if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t ev : e->join)
+        if (ev) cudaEventDestroy(ev);
+    if (e->fork) cudaEventDestroy(e->fork);
     if (e->own_stream) cudaStreamDestroy(e->own_stream);
     for (auto &t : e->tabs) dg_free_tables(t);
     delete e;
@@ -444,17 +487,10 @@ dg_status dg_ensemble_step(dg_ensemble e, int n)
             g.tile_rows = e->tile_rows;
             g.bps = e->bps;
             g.stream = e->stream;
-            int cur = e->cur;
-            const long long before = e->launches;
             ECUDA(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
-            dg_status st = DG_OK;
-            for (int k = 0; k < K && !st; ++k) {
-                st = launch_step(e, cur);
-                cur ^= 1;
-            }
+            dg_status st = launch_steps(e, K, e->cur);
             cudaGraph_t graph = nullptr;
             cudaError_t ce = cudaStreamEndCapture(e->stream, &graph);
-            e->launches = before;
             if (st) {
                 if (graph) cudaGraphDestroy(graph);
                 return st;
@@ -463,7 +499,7 @@ dg_status dg_ensemble_step(dg_ensemble e, int n)
             ce = cudaGraphInstantiate(&g.exec, graph, 0);
             cudaGraphDestroy(graph);
             if (ce != cudaSuccess) return efail(DG_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(ce));
-            g.cur_out = cur;
+            g.cur_out = e->cur ^ (K & 1);
             e->graphs.push_back(g);
             ge = &e->graphs.back();
         }
@@ -473,9 +509,10 @@ dg_status dg_ensemble_step(dg_ensemble e, int n)
             e->cur = ge->cur_out;
         }
     }
-    for (int k = 0; k < rest; ++k) {
-        if (dg_status st = launch_step(e, e->cur)) return st;
-        e->cur ^= 1;
+    if (rest) {
+        if (dg_status st = launch_steps(e, rest, e->cur)) return st;
+        e->launches += 3LL * rest;
+        e->cur ^= rest & 1;
     }
     unsigned st = 0;
     ECUDA(cudaMemcpyAsync(&st, e->d_status, sizeof st, cudaMemcpyDeviceToHost, e->stream));

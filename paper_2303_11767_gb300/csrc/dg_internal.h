@@ -110,7 +110,8 @@ struct StageArgs {
 };
 
 // Batched ensemble: the members' states are concatenated in every state
-// array; one persistent launch per stage walks a work list of tiles.
+// array; one persistent launch per stage and degree walks a work list of the
+// tiles of that degree.
 template <typename T>
 struct EnsMember {
     long long off;   // offset of the member's first value in the state arrays
@@ -120,7 +121,7 @@ struct EnsMember {
 };
 
 struct EnsItem {
-    int member, tx, ty, cost;
+    int member, tx, ty, n;
 };
 
 template <typename T>
@@ -141,7 +142,7 @@ struct EnsArgs {
 #define DG_ENS_TILE_ROWS_B 8
 
 template <typename T>
-int dg_launch_ensemble_stage(int tile_rows, int grid, const EnsArgs<T> &a, void *stream);
+int dg_launch_ensemble_stage(int tile_rows, int n, int grid, const EnsArgs<T> &a, void *stream);
 int dg_ensemble_tile_width(int n);   // elements per warp for degree n - 1
 
 // status bits written by device code

@@ -1,4 +1,4 @@
-"""Batched ensemble (one persistent launch per RK stage for meshes of uneven
+"""Batched ensemble (one persistent launch per RK stage and degree for meshes of uneven
 sizes and degrees): every member must evolve exactly as it does alone, and
 match the FP64 oracle within the FP32 tolerance."""
 import numpy as np
@@ -43,7 +43,7 @@ def test_members_match_single_mesh_solver_and_oracle(tile_rows):
         e.set_dt(dts)
         m0 = [e.total_mass(k) for k in range(len(MEMBERS))]
         e.step(nsteps)
-        assert e.stage_launches() == 3 * nsteps          # one launch per stage for all members
+        assert e.stage_launches() == 3 * nsteps          # RK stages of all members
         for k, (nlon_k, nlat_k, p) in enumerate(MEMBERS):
             got = e.get_state(k)
             want = oracles[k].step(states[k], nsteps, dts[k], 3)
@@ -71,3 +71,29 @@ def test_autotune_picks_a_valid_shape_and_restores_the_state():
             np.testing.assert_array_equal(e.get_state(k), before[k])
         e.step(4)                                         # the chosen shape runs
         assert all(np.isfinite(e.get_state(k)).all() for k in range(len(MEMBERS)))
+
+
+@pytest.mark.parametrize("degrees", [(3,), (2, 2), (0, 4), (4, 3, 2, 1, 0, 4)])
+@pytest.mark.parametrize("nsteps", [1, 7])
+def test_one_chain_of_launches_per_degree(degrees, nsteps):
+    """No fork, one, and all five degrees; steps in graphs of 4 and the rest, on the caller's stream."""
+    torch = pytest.importorskip("torch")
+    mesh = [(12 + 3 * k, 9 + k) for k in range(len(degrees))]
+    members = [(a, b, p) for (a, b), p in zip(mesh, degrees)]
+    stream = torch.cuda.Stream()
+    with dgswe.Ensemble(*zip(*members), R, G, OMEGA) as e:
+        e.set_option(dgswe.OPT_STREAM, stream.cuda_stream)
+        e.set_option(dgswe.OPT_STEPS_PER_GRAPH, 4)
+        states, dts = [], []
+        for k, (a, b, p) in enumerate(members):
+            o = O.Oracle.sphere(a, b, p, R, G, OMEGA)
+            u = o.project_tensor(synth.SmoothField(synth.ensemble_member_seed(k)).fields_grid)
+            states.append((o, u))
+            dts.append(o.max_dt(u, 0.1))
+            e.set_state(k, u)
+        e.set_dt(dts)
+        e.step(nsteps)
+        e.step(nsteps)
+        assert e.stage_launches() == 6 * nsteps
+        for k, (o, u) in enumerate(states):
+            assert _rel(e.get_state(k), o.step(u, 2 * nsteps, dts[k], 3)) < 1e-5
