@@ -312,7 +312,9 @@ __device__ __forceinline__ void put_chunk_split(unsigned char *p, uint32_t lo_of
 
 // ------------------------------------------------------------ stage kernel --
 
-template <int N, typename OpT, bool SPLIT>
+// KIND: the stage of SSP-RK3, compiled for what it reads and writes (0: no
+// increment yet; 1: increment in and out; 2: final), or -1: from the arguments.
+template <int N, typename OpT, bool SPLIT, int KIND>
 __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage_kernel(const StageArgs<float> A,
                                                                    const uint4 *__restrict__ gB1,
                                                                    const uint4 *__restrict__ gB2)
@@ -342,6 +344,10 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
     const int i = !lane_ok ? 0 : il < 0 ? il + A.nlon : il >= A.nlon ? il - A.nlon : il;
     const size_t rowlen = (size_t)3 * NP * A.nlon;
     const float href = A.href, gg = A.g;
+    const bool has_inc = KIND < 0 ? A.inc != nullptr : KIND > 0;
+    const bool fin = KIND < 0 ? A.out_base != nullptr : KIND == 2;
+    const bool has_lo = KIND < 0 ? A.lo != nullptr : KIND == 2;
+    const bool has_acc = KIND < 0 && A.acc_in;
     unsigned st = 0, st_int = 0;   // status of any thread / of interior elements only
     const uint32_t rowoff = (uint32_t)(32 * q4 + l) * 16;
     unsigned char *const opA = sm + SM::A;
@@ -385,7 +391,7 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
 #pragma unroll
             for (int k = 0; k < 8; ++k)
                 if (8 * c + k < NP) v[k] = __ldg(A.base + o0 + (size_t)k * A.nlon);
-            if (A.inc) {
+            if (has_inc) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
                     if (8 * c + k < NP) v[k] += __ldg(A.inc + o0 + (size_t)k * A.nlon);
@@ -397,8 +403,8 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
     };
     // the low parts and the RK4 accumulator are read only by the epilogue:
     // start moving this thread's share of them into L2 now
-    if (interior && (A.lo || A.acc_in)) {
-        const float *pl = A.lo ? A.lo : A.acc_in;
+    if (interior && (has_lo || has_acc)) {
+        const float *pl = has_lo ? A.lo : A.acc_in;
         const size_t o0 = (size_t)j * rowlen + i;
         for (int m = part; m < 3 * NP; m += TC_TPE)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(pl + o0 + (size_t)m * A.nlon));
@@ -754,7 +760,6 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
         constexpr int RPF = (N + TC_TPE - 1) / TC_TPE;   // rows per field and part, at most
         const size_t e0 = (size_t)j * rowlen + i;
         const float cdt = A.cc * A.dt, adt = A.ca * A.dt;
-        const bool fin = A.out_base != nullptr;
         float chk = 0.0f;   // non-finite tendency or state of an interior element: NaN (nf_acc)
 #pragma unroll 1
         for (int f = 0; f < 3; ++f) {
@@ -768,10 +773,10 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
 #pragma unroll
                 for (int a = 0; a < N; ++a) {
                     const size_t o = ob + (size_t)(a * A.nlon);
-                    vinc[rr][a] = ok && A.inc ? __ldg(A.inc + o) : 0.0f;
-                    vacc[rr][a] = ok && A.acc_in ? __ldg(A.acc_in + o) : 0.0f;
+                    vinc[rr][a] = ok && has_inc ? __ldg(A.inc + o) : 0.0f;
+                    vacc[rr][a] = ok && has_acc ? __ldg(A.acc_in + o) : 0.0f;
                     vbase[rr][a] = ok && fin ? __ldg(A.base + o) : 0.0f;
-                    vlo[rr][a] = ok && fin && A.lo ? __ldg(A.lo + o) : 0.0f;
+                    vlo[rr][a] = ok && fin && has_lo ? __ldg(A.lo + o) : 0.0f;
                 }
             }
             float r[8 * CN];
@@ -801,9 +806,9 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
                         const size_t o = ob + (size_t)(a * A.nlon);
                         const float kv = kk[a], inc = vinc[rr][a], acc = vacc[rr][a];
                         chk = dgk::nf_acc(kv, chk);
-                        if (A.out_rhs) A.out_rhs[o] = kv;
-                        if (A.inc_out) A.inc_out[o] = fmaf(cdt, kv, A.ci * inc);
-                        if (A.acc_out) A.acc_out[o] = fmaf(adt, kv, acc);
+                        if (KIND < 0 && A.out_rhs) A.out_rhs[o] = kv;
+                        if (KIND < 0 ? A.inc_out != nullptr : KIND < 2) A.inc_out[o] = fmaf(cdt, kv, A.ci * inc);
+                        if (KIND < 0 && A.acc_out) A.acc_out[o] = fmaf(adt, kv, acc);
                         if (fin) {
                             // u^{n+1} = (base + lo) + delta with an error-free two-sum
                             const float bs = vbase[rr][a], lo = vlo[rr][a];
@@ -814,7 +819,7 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
                             const float l1 = lo + err;
                             const float hi = s1 + l1;
                             A.out_base[o] = hi;
-                            if (A.out_lo) A.out_lo[o] = l1 - (hi - s1);
+                            if (KIND == 2 || A.out_lo) A.out_lo[o] = l1 - (hi - s1);
                             chk = dgk::nf_acc(hi, chk);
                         }
                     }
@@ -1038,9 +1043,10 @@ int prepare_tc(int op, TabSet &t)
     std::lock_guard<std::mutex> lock(g_tc_mu);
     if (tables_for<N, OpT>(dev, op, t)) return 1;
     if (!(g_attr[N - 1][op] >> dev & 1ull)) {
-        if (cudaFuncSetAttribute(tc_stage_kernel<N, OpT, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)SM::BYTES) != cudaSuccess)
-            return 1;
+        for (auto k : {tc_stage_kernel<N, OpT, SPLIT, -1>, tc_stage_kernel<N, OpT, SPLIT, 0>,
+                       tc_stage_kernel<N, OpT, SPLIT, 1>, tc_stage_kernel<N, OpT, SPLIT, 2>})
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::BYTES) != cudaSuccess)
+                return 1;
         g_attr[N - 1][op] |= 1ull << dev;
     }
     return 0;
@@ -1059,7 +1065,12 @@ int launch_tc(int op, const StageArgs<float> &a, cudaStream_t s)
         if (!t.b1 || !(g_attr[N - 1][op] >> dev & 1ull)) return 1;   // dg_prepare_stage_tc was not called
     }
     dim3 grid((a.nlon + TC_TW - 1) / TC_TW, (a.nlat + 3) / 4);
-    if (dgk::launch_pdl(tc_stage_kernel<N, OpT, SPLIT>, grid, dim3(128 * TC_TPE), SM::BYTES, s, a,
+    const bool plain = !a.out_rhs && !a.acc_in && !a.acc_out;
+    const auto k = plain && !a.inc && a.inc_out && !a.out_base && !a.lo           ? tc_stage_kernel<N, OpT, SPLIT, 0>
+                   : plain && a.inc && a.inc_out && !a.out_base && !a.lo          ? tc_stage_kernel<N, OpT, SPLIT, 1>
+                   : plain && a.inc && !a.inc_out && a.out_base && a.lo && a.out_lo ? tc_stage_kernel<N, OpT, SPLIT, 2>
+                                                                                    : tc_stage_kernel<N, OpT, SPLIT, -1>;
+    if (dgk::launch_pdl(k, grid, dim3(128 * TC_TPE), SM::BYTES, s, a,
                         (const uint4 *)t.b1, (const uint4 *)t.b2) != cudaSuccess)
         return 1;
     return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
