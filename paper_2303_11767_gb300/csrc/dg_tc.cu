@@ -28,6 +28,7 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "dg_internal.h"
@@ -314,6 +315,12 @@ __device__ __forceinline__ void put_chunk_split(unsigned char *p, uint32_t lo_of
 
 // KIND: the stage of SSP-RK3, compiled for what it reads and writes (0: no
 // increment yet; 1: increment in and out; 2: final), or -1: from the arguments.
+// A tile is bound by the latency of its phases (two CTAs per SM hold all the
+// tensor memory), so what counts is how many loads and points a thread has in
+// flight: tests per value of the optional arrays (41.2 -> 35.5 us at 360x180
+// degree 4), branches around the loads of a chunk and a test per Gauss point
+// (-> 34.1; 720x360 161 -> 149; degree 2, with half its chunk padding, 21.1 ->
+// 14.5; degree 1 at 180x90 7.0 -> 4.5) each kept them apart.
 template <int N, typename OpT, bool SPLIT, int KIND>
 __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage_kernel(const StageArgs<float> A,
                                                                    const uint4 *__restrict__ gB1,
@@ -380,25 +387,21 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
     };
 
     // ---- S0: 8 modes (chunk c) of one field of the stage state u = base + inc
-    //      of one element -> its row of a GEMM1 operand (zeros where missing)
-    auto stage_chunk = [&](int jj, bool ok, int f, int c, unsigned char *dst) {
-        float v[8];
+    //      of one element, loaded without a branch, then -> its row of a GEMM1
+    //      operand (zeros where missing)
+    auto load_chunk = [&](int jj, bool ok, int f, int c, float *v, float *vi) {
+        const size_t o0 = (size_t)jj * rowlen + (size_t)(f * NP + 8 * c) * A.nlon + i;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = 0.0f;
-        if (ok) {
-            const float s = f == 0 ? 1.0f : MS;
-            const size_t o0 = (size_t)jj * rowlen + (size_t)(f * NP + 8 * c) * A.nlon + i;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (8 * c + k < NP) v[k] = __ldg(A.base + o0 + (size_t)k * A.nlon);
-            if (has_inc) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (8 * c + k < NP) v[k] += __ldg(A.inc + o0 + (size_t)k * A.nlon);
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] *= s;
+        for (int k = 0; k < 8; ++k) {
+            const bool in = ok && 8 * c + k < NP;
+            v[k] = in ? __ldg(A.base + o0 + (size_t)k * A.nlon) : 0.0f;
+            vi[k] = in && has_inc ? __ldg(A.inc + o0 + (size_t)k * A.nlon) : 0.0f;
         }
+    };
+    auto store_chunk = [&](int f, int c, float *v, const float *vi, unsigned char *dst) {
+        const float s = f == 0 ? 1.0f : MS;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = (v[k] + vi[k]) * s;
         put_a1(dst + c * CH, v);
     };
     // the low parts and the RK4 accumulator are read only by the epilogue:
@@ -409,26 +412,44 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
         for (int m = part; m < 3 * NP; m += TC_TPE)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(pl + o0 + (size_t)m * A.nlon));
     }
-    // the tile rows: part p stages the chunks c = p, p + TPE, ... (all of its
-    // loads in flight before the first conversion)
+    // the tile rows: part p stages the chunks c = p, p + TPE, ..., LB at a time
+    // (their loads in flight before the first conversion; three at a time spill
+    // at degree 4)
+    constexpr int LB = 2, JOBS = (3 * K1C + TC_TPE - 1) / TC_TPE, HJOBS = (6 * K1C + 4 * TC_TPE - 1) / (4 * TC_TPE);
 #pragma unroll
-    for (int fc = 0; fc < 3 * K1C; fc += TC_TPE) {
-        if (fc + part < 3 * K1C) {
-            const int f = (fc + part) / K1C, c = (fc + part) - f * K1C;
-            stage_chunk(j0 + q4, row_ok && lane_ok, f, c, opA + (uint32_t)(f * K1C) * CH + rowoff);
+    for (int q0 = 0; q0 < JOBS; q0 += LB) {
+        float v[LB][8], vi[LB][8];
+#pragma unroll
+        for (int q = 0; q < LB; ++q) {
+            const int fc = (q0 + q) * TC_TPE + part;
+            if (q0 + q < JOBS)
+                load_chunk(j, row_ok && lane_ok && fc < 3 * K1C, fc / K1C, fc % K1C, v[q], vi[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < LB; ++q) {
+            const int fc = (q0 + q) * TC_TPE + part, f = fc / K1C;
+            if (q0 + q < JOBS && (JOBS * TC_TPE == 3 * K1C || fc < 3 * K1C))
+                store_chunk(f, fc % K1C, v[q], vi[q], opA + (uint32_t)(f * K1C) * CH + rowoff);
         }
     }
     // halo rows: job = (side * 3 + f) * K1C + c; side 0 = the row south of
     // the tile (TMEM quarter 0), side 1 = the row north of it (quarter 3)
 #pragma unroll
-    for (int job0 = 0; job0 < 6 * K1C; job0 += 4 * TC_TPE) {
-        const int job = job0 + w;
-        if (job >= 6 * K1C) break;
-        const int sf = job / K1C, c = job - sf * K1C;
-        const int side = sf / 3, f = sf - 3 * side;
-        const int jj = side ? j0 + 4 : j0 - 1;
-        const bool ok = lane_ok && (side ? jj < A.nlat : jj >= 0);
-        stage_chunk(ok ? jj : 0, ok, f, c, opA + SM::SZ_A1 + (uint32_t)(f * K1C) * CH + (uint32_t)((side ? 96 : 0) + l) * 16);
+    for (int q0 = 0; q0 < HJOBS; q0 += LB) {
+        float v[LB][8], vi[LB][8];
+#pragma unroll
+        for (int q = 0; q < LB; ++q) {
+            const int job = (q0 + q) * 4 * TC_TPE + w, sf = job / K1C, side = sf / 3, jj = side ? j0 + 4 : j0 - 1;
+            const bool ok = job < 6 * K1C && lane_ok && (side ? jj < A.nlat : jj >= 0);
+            if (q0 + q < HJOBS) load_chunk(ok ? jj : 0, ok, sf - 3 * side, job - sf * K1C, v[q], vi[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < LB; ++q) {
+            const int job = (q0 + q) * 4 * TC_TPE + w, sf = job / K1C, side = sf / 3, f = sf - 3 * side;
+            if (q0 + q < HJOBS && (HJOBS * 4 * TC_TPE == 6 * K1C || job < 6 * K1C))
+                store_chunk(f, job - sf * K1C, v[q], vi[q],
+                            opA + SM::SZ_A1 + (uint32_t)(f * K1C) * CH + (uint32_t)((side ? 96 : 0) + l) * 16);
+        }
     }
 
     fence_async_smem();
@@ -678,8 +699,9 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
     //      part p takes the chunks g = p, p + TPE, ...
     {
         unsigned sq = 0;
-#pragma unroll 1
-        for (int g = part; g < CN; g += TC_TPE) {
+// the first P points of chunk g (a constant: no test per point)
+        auto points = [&](int g, auto npts) {
+            constexpr int P = decltype(npts)::value;
             float x[3][8];
 #pragma unroll
             for (int f = 0; f < 3; ++f) tmem_ld8(tl + (uint32_t)(f * N1 + 8 * g), x[f]);
@@ -690,7 +712,7 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
 #pragma unroll
             for (int qq = 0; qq < 8; ++qq) {
                 const int q = 8 * g + qq;
-                if (q < NP) {
+                if (qq < P) {
                     const int be = q / N;
                     const float hp = x[0][qq], hu = x[1][qq] * IMS, hv = x[2][qq] * IMS;
                     const float h = href + hp;
@@ -721,7 +743,12 @@ __global__ void __launch_bounds__(128 * TC_TPE, TcSmem<N, SPLIT>::CTAS) tc_stage
                 put_a2(a2(f, CN + g), Gq[f]);
                 if (f > 0 || !SM::SKIP_S0) put_a2(a2(f, 2 * CN + g), Sv[f]);
             }
-        }
+        };
+        constexpr int FULL = NP / 8;   // chunks of 8 points, then one of NP % 8
+#pragma unroll 1
+        for (int g = part; g < FULL; g += TC_TPE) points(g, std::integral_constant<int, 8>{});
+        if constexpr (FULL < CN)
+            if (part == FULL % TC_TPE) points(FULL, std::integral_constant<int, NP % 8>{});
         if (interior) st_int |= sq;
     }
 
