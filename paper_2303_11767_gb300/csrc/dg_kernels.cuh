@@ -1170,7 +1170,7 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // One thread per element where the mesh has enough elements for it; else
     // N lanes per element, whose tiles have the shorter chain (one tile takes
     // 8 instead of 13 us at degree 4).  The line lies where both take the same
-    // time; us per stage, lanes / threads: degree 4 160x80 10.9 / 13.1, 200x100
+    // time; us per stage, lanes / threads: degree 4 160x80 10.2 / 13.1, 200x100
     // 14.2 / 14.5, 240x120 19.8 / 14.6, 360x180 40.5 / 30.1, 1440x720 586 / 373;
     // degree 3 220x110 7.3 / 9.4, 260x130 10.2 / 9.6, 360x180 16.5 / 14.4,
     // 1440x720 235 / 202; degree 2 180x90 6.6 / 6.3, 220x110 8.0 / 6.7, 720x360
@@ -1218,29 +1218,38 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // 74.7 65.3; 240x120 degree 2 124 113 104 127 141, degree 1 60.9 50.6 62.0
     // 45.4 65.4; 300x150 degree 0 39.9 32.4 25.3 29.2 29.0.  Heights 6 and 3 win
     // nowhere by more than 3 % (360x180 degree 3 362 against 370), one row never.
-    // FP32 takes 8 rows (90x45 degree 3 4.5, 4 rows 4.7; 180x90 5.9 6.2).
-    if constexpr (sizeof(T) == 8) {
-        constexpr int rows[] = {8, 7, 5, 4, 2};
-        constexpr double cost[] = {1.0, 1.02, 1.03, 1.04, 1.2};
+    //
+    // FP32, bound by the latency of its phases and the issue slots, takes 8, 5
+    // or 4 rows by the same count; at 8, 5, 4 rows: 20x10 degree 2 4.65 4.31
+    // 4.06; 120x60 degree 2 4.97 4.55 4.75; 150x75 degree 2 5.05 5.19 4.87;
+    // 90x45 degree 4 8.0 7.0 7.4; 120x60 degree 4 9.3 8.3 7.8; 160x80 degree 4
+    // 10.9 10.2 10.7; 72x36 degree 3 4.49 4.45 4.11; 180x90 degree 3 5.87 5.98
+    // 6.11; 200x100 degree 3 7.1 6.8 6.7; 180x90 degree 1 3.52 3.72 3.61; 240x120
+    // degree 1 4.06 4.07 3.98.  It counts the whole mesh's rows, as above.
+    {
+        constexpr bool F64 = sizeof(T) == 8;
+        constexpr int rows[] = {8, 5, 4, 7, 2}, choices = F64 ? 5 : 3;
+        constexpr double cost[] = {1.0, F64 ? 1.03 : N == 5 ? 0.95 : N == 3 ? 1.0 : 1.08,
+                                   F64 ? 1.04 : N == 5 || N == 3 ? 0.97 : 1.03, 1.02, 1.2};
+        const int nlat = F64 ? a.nlat : a.nlat_mesh;
         int w = DG_WARPS;
         double best = 0;
-        for (int c = 0; c < 5; ++c) {
-            const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((a.nlat + rows[c] - 1) / rows[c]);
+        for (int c = 0; c < choices; ++c) {
+            const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((nlat + rows[c] - 1) / rows[c]);
             const long long per_sm = (tiles + DG_SMS - 1) / DG_SMS * rows[c];
-            const double quarter = 3.5 * (double)((per_sm + 3) / 4);
+            const double quarter = F64 ? 3.5 * (double)((per_sm + 3) / 4) : 0;
             const double work = cost[c] * (quarter > (double)per_sm ? quarter : (double)per_sm);
             if (c == 0 || work < best) {
                 best = work;
                 w = rows[c];
             }
         }
-        switch (w) {
-        case 2: return launch_stage_w<T, N, 2>(a, s);
-        case 4: return launch_stage_w<T, N, 4>(a, s);
-        case 5: return launch_stage_w<T, N, 5>(a, s);
-        case 7: return launch_stage_w<T, N, 7>(a, s);
-        default: break;
+        if constexpr (F64) {
+            if (w == 2) return launch_stage_w<T, N, 2>(a, s);
+            if (w == 7) return launch_stage_w<T, N, 7>(a, s);
         }
+        if (w == 4) return launch_stage_w<T, N, 4>(a, s);
+        if (w == 5) return launch_stage_w<T, N, 5>(a, s);
     }
     return launch_stage_w<T, N, DG_WARPS>(a, s);
 }

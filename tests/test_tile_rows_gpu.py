@@ -1,9 +1,11 @@
 """The FP64 stage at every tile height its launch rule takes (8, 7, 5, 4, 2 rows;
-launch_stage_n in csrc/dg_kernels.cuh), on meshes with ragged last tiles, its
+launch_stage_n in csrc/dg_kernels.cuh), on meshes with ragged last tiles, the
+FP32 stage at the short ones (5, 4 rows), the FP64 stage's
 one-lane-per-point kernel (csrc/dg_stage_f64pt.cuh) on the meshes below its line
 (every RK kind, the status bits, bands, the global alpha), and the planar
 shallow-water problem on both.  Tolerances as in
-test_parity_gpu.py (tendencies, 3e-14 of the magnitude bound) and
+test_parity_gpu.py (tendencies, 3e-14 or 1e-6 of the magnitude bound; FP32
+states 1e-5) and
 test_plane_gpu.py (1e-12)."""
 import numpy as np
 import pytest
@@ -105,3 +107,32 @@ def test_tile_rows_bands_get_the_whole_mesh_bits(p, nlon, nlat, rows):
     dt = o.max_dt(u, 0.1)
     whole = _whole(u, nlon, nlat, p, "fp64", 2, dt, 3, torch)[0]
     assert np.array_equal(_run_bands(u, nlon, nlat, p, "fp64", 3, 2, dt, 3, torch)[0], whole)
+
+
+def tile_rows_f32(nlon, nlat, n):
+    """The launch rule."""
+    rows, best = 8, None
+    for c, cost in ((8, 1.0), (5, 0.95 if n == 5 else 1.0 if n == 3 else 1.08), (4, 0.97 if n in (3, 5) else 1.03)):
+        work = cost * c * -(-(-(-nlon // (32 // n)) * -(-nlat // c)) // SMS)
+        if best is None or work < best:
+            rows, best = c, work
+    return rows
+
+
+F32 = [(0, 162, 37, 4), (0, 206, 93, 5), (1, 7, 15, 4), (1, 141, 67, 5), (2, 16, 46, 4), (2, 157, 43, 5), (3, 23, 9, 4), (3, 217, 44, 5), (4, 85, 44, 5), (4, 133, 69, 4)]
+
+
+@pytest.mark.parametrize("p,nlon,nlat,rows", F32)
+def test_short_fp32_tiles(p, nlon, nlat, rows):
+    torch = pytest.importorskip("torch")
+    assert tile_rows_f32(nlon, nlat, p + 1) == rows
+    o, u = case(nlon, nlat, p, 11)
+    with dgswe.Solver(nlon, nlat, p, precision="fp32") as s:
+        k = s.rhs(u)
+    what = f"rhs p={p} {nlon}x{nlat} fp32, {rows} tile rows"
+    assert_within(tend_err(k, o.rhs(u), o.rhs_magnitude(u), what), 1e-6, what)
+    dt = o.max_dt(u, 0.1)
+    for order in (3, 4):
+        whole = _whole(u, nlon, nlat, p, "fp32", 3, dt, order, torch)[0]
+        assert_within(state_err(whole, o.step(u, 3, dt, order)), 1e-5, what)
+    assert np.array_equal(_run_bands(u, nlon, nlat, p, "fp32", 2, 3, dt, 4, torch)[0], whole)
