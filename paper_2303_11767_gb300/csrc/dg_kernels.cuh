@@ -21,10 +21,12 @@
 // Thread mapping: one warp owns G = 32 / N consecutive elements of one
 // latitude row; N lanes per element.  Lane k first owns row b = k of the modal
 // coefficients, then column alpha = k of the Gauss points (after a transpose
-// through shared memory), then row b = k again for the output.  A block of
-// DG_WARPS warps covers G x DG_WARPS elements.  Up to p = 3 there is one
-// kernel per stage kind (increment or not, final stage or not) and the FP32
-// contractions run on paired FP32 instructions.
+// through shared memory), then row b = k again for the output.  A block of W
+// warps covers G x W elements.  Up to p = 3 there is one kernel per stage kind
+// (increment or not, final stage or not) and the FP32 contractions run on
+// paired FP32 instructions.  Large FP32 meshes run one thread per element
+// (dg_stage_ept.cuh) and small FP64 meshes one lane per Gauss point
+// (dg_stage_f64pt.cuh) instead; launch_stage_n holds the lines.
 #pragma once
 
 #include <cuda_runtime.h>
