@@ -1602,7 +1602,7 @@ __global__ void max_speed_kernel(const T *__restrict__ u, int nel, double href, 
     const BasisTab<T> &B = c_basis[N - 1];
     const int lane = threadIdx.x & 31, e0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
     const float lo = __uint_as_float(*lower);
-    unsigned todo = __ballot_sync(0xffffffffu, e0 + lane < nel && !(upper[min(e0 + lane, nel - 1)] < lo));
+    unsigned todo = __ballot_sync(0xffffffffu, e0 + lane < nel && (!upper || !(upper[min(e0 + lane, nel - 1)] < lo)));
     double best = 0.0;
     unsigned st = 0;
     constexpr int EPW = 32 / (N * N);   // elements at a time
@@ -1826,6 +1826,14 @@ int dg_launch_max_speed<DG_REAL>(const DG_REAL *u, int nlon, int nlat, int n, do
 #define DG_MS(NN)                                                                                                     \
     dgk::speed_bound_kernel<DG_REAL, NN><<<bb, dgk::SPEED_THREADS, 0, s>>>(u, nel, (float)href, (float)g, upper, lower); \
     dgk::max_speed_kernel<DG_REAL, NN><<<blocks, threads, 0, s>>>(u, nel, href, g, upper, lower, maxbits, status)
+    // At degree 0 a warp's 32 points are one short FP64 chain, less than the bound
+    // pass and its launch until several warps share an SM quarter (dg_max_dt in us
+    // without / with the bound pass: 16x8 26.4 / 37.2, 180x90 26.3 / 37.2, 360x180
+    // 35.7 / 38.0, 500x250 39.8 / 38.0, 720x360 53.2 / 38.9).
+    if (n == 1 && nel <= 98304) {
+        dgk::max_speed_kernel<DG_REAL, 1><<<blocks, threads, 0, s>>>(u, nel, href, g, nullptr, lower, maxbits, status);
+        return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
+    }
     switch (n) {
     case 1: DG_MS(1); break;
     case 2: DG_MS(2); break;

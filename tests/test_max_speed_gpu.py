@@ -34,7 +34,7 @@ def _state(kind, nlon, nlat, p, rng):
 
 
 @pytest.mark.parametrize("kind", ["rest", "rough", "one", "shallow", "close"])
-@pytest.mark.parametrize("nlon,nlat,p", [(37, 21, 0), (33, 19, 1), (29, 23, 2), (31, 18, 3), (27, 17, 4), (5, 3, 4)])
+@pytest.mark.parametrize("nlon,nlat,p", [(37, 21, 0), (33, 19, 1), (29, 23, 2), (31, 18, 3), (27, 17, 4), (5, 3, 4), (401, 247, 0)])
 def test_max_dt_matches_oracle(nlon, nlat, p, kind):
     u = _state(kind, nlon, nlat, p, np.random.default_rng(nlon + p))
     want = O.Oracle.sphere(nlon, nlat, p, R, G, OMEGA).max_dt(u, 0.1)
