@@ -1511,7 +1511,10 @@ static __global__ void __launch_bounds__(MASS_THREADS) mass_final_kernel(const d
 // S = sum |m| max|L_a| max|L_b| in size, and carries at most 2 N + 4 < 16
 // roundings, so its error is below 2^-20 S; 2^-19 is used.  A point whose
 // depth is not surely positive, and anything non-finite, goes to the FP64 pass,
-// which reports it.  dg_max_dt at 1440x720 degree 4: 10.0 -> 0.28 ms
+// which reports it.  Values below FP32's normal range lose up to 2^-149 each, so a
+// point value is taken to be off by 2^-120 more, and a momentum by 2^-70 (its
+// square is lost below 2^-149); where g h itself comes near that range the element
+// is evaluated.  dg_max_dt at 1440x720 degree 4: 10.0 -> 0.28 ms
 // (a fluid at rest, where every element ties: 11.2 -> 7.3 ms).
 constexpr int SPEED_THREADS = 64;
 
@@ -1556,7 +1559,7 @@ __global__ void __launch_bounds__(SPEED_THREADS) speed_bound_kernel(const T *__r
                 }
                 sum = fmaf(row, lmax[b], sum);
             }
-            err[f] = sum * 0x1p-19f;
+            err[f] = fmaf(sum, 0x1p-19f, 0x1p-120f);
 #pragma unroll
             for (int p = 0; p < N; ++p)
 #pragma unroll
@@ -1567,7 +1570,7 @@ __global__ void __launch_bounds__(SPEED_THREADS) speed_bound_kernel(const T *__r
                     q[f][p][r] = v;
                 }
         }
-        const float em = 1.5f * fmaxf(err[1], err[2]);
+        const float em = fmaf(1.5f, fmaxf(err[1], err[2]), 0x1p-70f);
         float up = 0.f;
 #pragma unroll
         for (int p = 0; p < N; ++p)
@@ -1578,7 +1581,7 @@ __global__ void __launch_bounds__(SPEED_THREADS) speed_bound_kernel(const T *__r
                 const float mom = sqrtf(fmaf(q[1][p][r], q[1][p][r], q[2][p][r] * q[2][p][r]));
                 const float us = ((mom + em) / hl + sqrtf(g * hh)) * 1.00001f;
                 // (a comparison that fails on NaN: the element is left to the FP64 pass)
-                if (!(hl > 0.f) || !(us < 3.0e38f)) up = INFINITY;
+                if (!(hl > 0.f) || !(us < 3.0e38f) || !(g * hl > 0x1p-100f)) up = INFINITY;
                 else {
                     up = fmaxf(up, us);
                     lo = fmaxf(lo, (fmaxf(mom - em, 0.f) / hh + sqrtf(g * hl)) * 0.99999f);

@@ -62,3 +62,18 @@ def test_bad_depth_is_reported(j, i, prec):
         with pytest.raises(dgswe.DGError) as e:
             s.max_dt(0.1)
         assert e.value.status == dgswe.DG_ENONPHYSICAL
+
+
+@pytest.mark.parametrize("p", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("h,u,deep", [(1e-27, 500.0, 1000.0), (1e-27, 500.0, 1e-22), (1e-40, 300.0, 10.0), (1e-33, 4e-4, 1e-30)])
+def test_thin_fast_element(p, h, u, deep):
+    """One element whose depth and momentum, or the momentum's square, lie below
+    FP32's range, faster than the others."""
+    nlon, nlat = (401, 247) if p == 0 else (23, 17)
+    s = np.zeros((nlat, nlon, 3, (p + 1) ** 2))
+    s[..., 0, 0] = 2.0 * deep
+    s[5, 7, 0, 0], s[5, 7, 1, 0] = 2.0 * h, 2.0 * h * u
+    want = O.Oracle.sphere(nlon, nlat, p, R, G, OMEGA).max_dt(s, 0.1)
+    with dgswe.Solver(nlon, nlat, p, precision="fp64") as solver:
+        solver.set_state(s)
+        assert abs(solver.max_dt(0.1) / want - 1) < 1e-12
