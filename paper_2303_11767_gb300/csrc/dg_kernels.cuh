@@ -1200,10 +1200,10 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
 #ifndef DG_REAL_IS_F32
     // One lane per Gauss point on small meshes: up to 9 to 14 of its warps per
     // SM, where both take the same time.  us per stage, tiles / points: degree 1
-    // 20x10 20.7 / 11.8, 120x60 21.2 / 16.3, 180x90 31.5 / 35.2; degree 2 60x30
-    // 28.8 / 14.4, 90x45 28.6 / 26.3, 120x60 38 / 53; degree 3 50x50 36.3 / 23.7,
-    // 90x45 36.4 / 34.3, 120x60 52 / 65; degree 4 50x25 47.5 / 26.0, 72x36 47 /
-    // 55.  (The whole mesh's rows: a band runs the whole mesh's kernel.)
+    // 20x10 22.2 / 13.0, 120x60 22.6 / 17.4, 180x90 33.1 / 38.0; degree 2 60x30
+    // 29.9 / 15.3, 90x45 30.0 / 28.1, 120x60 40.5 / 56.6; degree 3 50x50 37.9 / 24.7,
+    // 90x45 38.0 / 35.8, 120x60 53.0 / 68.3; degree 4 50x25 48.0 / 26.9, 72x36 48.1 /
+    // 58.4.  (The whole mesh's rows: a band runs the whole mesh's kernel.)
     if constexpr (N >= 2) {
         constexpr long long most = N == 2 ? 14500 : N == 3 ? 4100 : N == 4 ? 4250 : 2100;
         if ((long long)a.nlon * a.nlat_mesh <= most) return launch_pt_n<N>(a, s);
@@ -1215,11 +1215,11 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // the SM with one warp more than the others counts 3.5 rows per warp: a
     // single tile of 5 rows takes as long as one of 7.  Measured at 8, 7, 5, 4,
     // 2 rows (us per stage; more heights to choose from, fewer SMs that wait):
-    // 180x90 degree 3 108 102 112 115 132; 120x60 degree 3 53.7 50.6 71.2 58.1
-    // 52.1; 360x180 degree 4 692 693 651 648 725; 90x45 degree 4 71.6 64.7 70.8
-    // 74.7 65.3; 240x120 degree 2 124 113 104 127 141, degree 1 60.9 50.6 62.0
-    // 45.4 65.4; 300x150 degree 0 39.9 32.4 25.3 29.2 29.0.  Heights 6 and 3 win
-    // nowhere by more than 3 % (360x180 degree 3 362 against 370), one row never.
+    // 180x90 degree 3 111 105 115 119 136; 120x60 degree 3 55.7 53.0 74.5 60.9
+    // 54.3; 360x180 degree 4 718 723 685 674 755; 90x45 degree 4 74.6 67.4 74.2
+    // 77.9 68.1; 240x120 degree 2 131 120 110 133 149, degree 1 65.3 52.4 64.9
+    // 48.9 70.4; 300x150 degree 0 43.6 34.9 28.0 32.4 32.7.  Heights 6 and 3 won
+    // nowhere by more than 3 %, one row never.
     //
     // FP32, bound by the latency of its phases and the issue slots, takes 8, 5
     // or 4 rows by the same count; at 8, 5, 4 rows: 20x10 degree 2 4.65 4.31

@@ -7,7 +7,7 @@
 // independent the operations are.  On a mesh with less than a warp per quarter
 // the stage therefore takes (FP64 instructions of a warp) x 64 cycles, and
 // lanes are free: with N lanes per element (stage_tile) a warp has some 600 to
-// 1000 of them, with N^2 lanes 250.  A warp here holds 32 / N^2 elements and
+// 1000 of them, with N^2 lanes about 300.  A warp here holds 32 / N^2 elements and
 // depends on no other warp: it evaluates its elements' four edges itself, from
 // its own and the four neighbours' modes (a third more operations in all, so
 // the tiles win on meshes that fill the chip; the line is at launch_stage_n).
