@@ -1213,12 +1213,18 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // x rows x the cost of a row in a tile of that height (a short tile has more
     // ring traces and evaluates more of its boundary edges twice).  A quarter of
     // the SM with one warp more than the others counts 3.5 rows per warp: a
-    // single tile of 5 rows takes as long as one of 7.  Measured at 8, 7, 5, 4,
+    // single tile of 5 rows takes as long as one of 7.  At degrees 0 and 1 it is the
+    // rows alone, and at degree 0 a single round of 7-row tiles shares SMs from about
+    // 95 tiles on.  Costs of a row per degree are fitted to the 61 sizes of 16x9 to
+    // 1100x550 (the height taken is on average 0.2 to 0.5 % and at most 6 % slower than
+    // the best one).  Measured at 8, 7, 5, 4,
     // 2 rows (us per stage; more heights to choose from, fewer SMs that wait):
     // 180x90 degree 3 111 105 115 119 136; 120x60 degree 3 55.7 53.0 74.5 60.9
     // 54.3; 360x180 degree 4 718 723 685 674 755; 90x45 degree 4 74.6 67.4 74.2
     // 77.9 68.1; 240x120 degree 2 131 120 110 133 149, degree 1 65.3 52.4 64.9
-    // 48.9 70.4; 300x150 degree 0 43.6 34.9 28.0 32.4 32.7.  Heights 6 and 3 won
+    // 48.9 70.4; 300x150 degree 0 43.6 34.9 28.0 32.4 32.7; 248x124 degree 0 22.3
+    // 28.3 28.0 23.4 26.5; 360x179 degree 0 43.9 46.3 54.0 62.4 51.8; 543x271 degree
+    // 1 259 233 252 259 287; 181x87 degree 2 87.4 80.0 93.7 89.8 99.5.  Heights 6 and 3 won
     // nowhere by more than 3 %, one row never.
     //
     // FP32, bound by the latency of its phases and the issue slots, takes 8, 5
@@ -1231,15 +1237,17 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     {
         constexpr bool F64 = sizeof(T) == 8;
         constexpr int rows[] = {8, 5, 4, 7, 2}, choices = F64 ? 5 : 3;
-        constexpr double cost[] = {1.0, F64 ? 1.03 : N == 5 ? 0.95 : N == 3 ? 1.0 : 1.08,
-                                   F64 ? 1.04 : N == 5 || N == 3 ? 0.97 : 1.03, 1.02, 1.2};
+        constexpr double cost[] = {1.0, F64 ? (N <= 2 ? 1.1 : 1.03) : N == 5 ? 0.95 : N == 3 ? 1.0 : 1.08,
+                                   F64 ? (N == 1 ? 1.08 : N == 3 ? 1.2 : 1.04) : N == 5 || N == 3 ? 0.97 : 1.03,
+                                   N <= 2 ? 0.96 : N == 3 ? 1.0 : 1.02, 1.2};
         const int nlat = F64 ? a.nlat : a.nlat_mesh;
         int w = DG_WARPS;
         double best = 0;
         for (int c = 0; c < choices; ++c) {
             const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((nlat + rows[c] - 1) / rows[c]);
             const long long per_sm = (tiles + DG_SMS - 1) / DG_SMS * rows[c];
-            const double quarter = F64 ? 3.5 * (double)((per_sm + 3) / 4) : 0;
+            if (F64 && N == 1 && rows[c] == 7 && tiles <= DG_SMS) continue;
+            const double quarter = F64 && N >= 3 ? 3.5 * (double)((per_sm + 3) / 4) : 0;
             const double work = cost[c] * (quarter > (double)per_sm ? quarter : (double)per_sm);
             if (c == 0 || work < best) {
                 best = work;

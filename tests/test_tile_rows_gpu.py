@@ -23,16 +23,19 @@ SMS = 152
 def tile_rows(nlon, nlat, n):
     """The launch rule."""
     rows, best = 8, None
-    for c, cost in ((8, 1.0), (7, 1.02), (5, 1.03), (4, 1.04), (2, 1.2)):
+    costs = {1: (1.0, 1.1, 1.08, 0.96, 1.2), 2: (1.0, 1.1, 1.04, 0.96, 1.2), 3: (1.0, 1.03, 1.2, 1.0, 1.2)}
+    for c, cost in zip((8, 5, 4, 7, 2), costs.get(n, (1.0, 1.03, 1.04, 1.02, 1.2))):
         tiles = -(-nlon // (32 // n)) * -(-nlat // c)
+        if n == 1 and c == 7 and tiles <= SMS:
+            continue
         per_sm = -(-tiles // SMS) * c
-        work = cost * max(per_sm, 3.5 * (-(-per_sm // 4)))
+        work = cost * (max(per_sm, 3.5 * (-(-per_sm // 4))) if n >= 3 else per_sm)
         if best is None or work < best:
             rows, best = c, work
     return rows
 
 
-MESHES = [(0, 122, 34, 4), (0, 190, 122, 7), (0, 241, 139, 8), (0, 194, 85, 2), (0, 259, 137, 5), (1, 231, 79, 8), (1, 148, 137, 5), (1, 231, 103, 4), (1, 156, 100, 7), (1, 131, 133, 2), (2, 55, 87, 4), (2, 199, 40, 7), (2, 131, 89, 5), (2, 107, 100, 8), (2, 216, 25, 2), (3, 52, 138, 7), (3, 169, 67, 4), (3, 189, 92, 5), (3, 147, 123, 8), (3, 162, 113, 2), (4, 149, 59, 5), (4, 81, 58, 7), (4, 203, 29, 8), (4, 125, 113, 2), (4, 89, 25, 4)]
+MESHES = [(0, 122, 34, 2), (0, 190, 122, 5), (0, 65, 101, 4), (0, 340, 167, 7), (0, 241, 139, 8), (0, 194, 85, 2), (0, 259, 137, 5), (1, 231, 79, 8), (1, 148, 137, 5), (1, 231, 103, 4), (1, 156, 100, 7), (1, 131, 133, 2), (2, 55, 87, 4), (2, 199, 40, 7), (2, 131, 89, 5), (2, 107, 100, 8), (2, 216, 25, 2), (3, 52, 138, 7), (3, 169, 67, 4), (3, 189, 92, 5), (3, 147, 123, 8), (3, 162, 113, 2), (4, 149, 59, 5), (4, 81, 58, 7), (4, 203, 29, 8), (4, 125, 113, 2), (4, 89, 25, 4)]
 
 
 @pytest.mark.parametrize("p,nlon,nlat,rows", MESHES)
