@@ -1233,10 +1233,15 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // 90x45 degree 4 8.0 7.0 7.4; 120x60 degree 4 9.3 8.3 7.8; 160x80 degree 4
     // 10.9 10.2 10.7; 72x36 degree 3 4.49 4.45 4.11; 180x90 degree 3 5.87 5.98
     // 6.11; 200x100 degree 3 7.1 6.8 6.7; 180x90 degree 1 3.52 3.72 3.61; 240x120
-    // degree 1 4.06 4.07 3.98.  It counts the whole mesh's rows, as above.
+    // degree 1 4.06 4.07 3.98.  Short tiles over many rounds lose more than they
+    // save (200x100 degree 4, 3 / 5 / 6 rounds: 14.2 16.8 16.3), so they are taken up
+    // to 20 rows per SM; at degree 0, where one round takes the same time at every
+    // height (180x90 2.87 2.96 3.07; 500x250 5.65 5.70 5.92), only 5 rows instead of
+    // two rounds of 8 (300x150 3.37 3.18 3.35), and at degree 1 no 5 rows where 8 take
+    // one round (150x74 3.46 3.58).  It counts the whole mesh's rows, as above.
     {
         constexpr bool F64 = sizeof(T) == 8;
-        constexpr int rows[] = {8, 5, 4, 7, 2}, choices = F64 ? 5 : 3;
+        constexpr int rows[] = {8, 5, 4, 7, 2}, choices = F64 ? 5 : N == 1 ? 2 : 3;
         constexpr double cost[] = {1.0, F64 ? (N <= 2 ? 1.1 : 1.03) : N == 5 ? 0.95 : N == 3 ? 1.0 : 1.08,
                                    F64 ? (N == 1 ? 1.08 : N == 3 ? 1.2 : 1.04) : N == 5 || N == 3 ? 0.97 : 1.03,
                                    N <= 2 ? 0.96 : N == 3 ? 1.0 : 1.02, 1.2};
@@ -1247,6 +1252,8 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
             const long long tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((nlat + rows[c] - 1) / rows[c]);
             const long long per_sm = (tiles + DG_SMS - 1) / DG_SMS * rows[c];
             if (F64 && N == 1 && rows[c] == 7 && tiles <= DG_SMS) continue;
+            if (!F64 && c > 0 && per_sm > (N == 1 ? 10 : 20)) continue;
+            if (!F64 && N <= 2 && rows[c] == 5 && best <= 8) continue;   // (8 rows take one round)
             const double quarter = F64 && N >= 3 ? 3.5 * (double)((per_sm + 3) / 4) : 0;
             const double work = cost[c] * (quarter > (double)per_sm ? quarter : (double)per_sm);
             if (c == 0 || work < best) {
@@ -1258,7 +1265,9 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
             if (w == 2) return launch_stage_w<T, N, 2>(a, s);
             if (w == 7) return launch_stage_w<T, N, 7>(a, s);
         }
-        if (w == 4) return launch_stage_w<T, N, 4>(a, s);
+        if constexpr (F64 || N >= 2) {
+            if (w == 4) return launch_stage_w<T, N, 4>(a, s);
+        }
         if (w == 5) return launch_stage_w<T, N, 5>(a, s);
     }
     return launch_stage_w<T, N, DG_WARPS>(a, s);

@@ -115,14 +115,17 @@ def test_tile_rows_bands_get_the_whole_mesh_bits(p, nlon, nlat, rows):
 def tile_rows_f32(nlon, nlat, n):
     """The launch rule."""
     rows, best = 8, None
-    for c, cost in ((8, 1.0), (5, 0.95 if n == 5 else 1.0 if n == 3 else 1.08), (4, 0.97 if n in (3, 5) else 1.03)):
-        work = cost * c * -(-(-(-nlon // (32 // n)) * -(-nlat // c)) // SMS)
+    for c, cost in ((8, 1.0), (5, 0.95 if n == 5 else 1.0 if n == 3 else 1.08), (4, 0.97 if n in (3, 5) else 1.03))[:2 if n == 1 else 3]:
+        per_sm = c * -(-(-(-nlon // (32 // n)) * -(-nlat // c)) // SMS)
+        if c < 8 and (per_sm > (10 if n == 1 else 20) or n <= 2 and c == 5 and best <= 8):
+            continue
+        work = cost * per_sm
         if best is None or work < best:
             rows, best = c, work
     return rows
 
 
-F32 = [(0, 162, 37, 4), (0, 206, 93, 5), (1, 7, 15, 4), (1, 141, 67, 5), (2, 16, 46, 4), (2, 157, 43, 5), (3, 23, 9, 4), (3, 217, 44, 5), (4, 85, 44, 5), (4, 133, 69, 4)]
+F32 = [(0, 162, 37, 8), (0, 206, 93, 8), (0, 299, 149, 5), (4, 196, 97, 8), (1, 7, 15, 4), (1, 141, 67, 8), (1, 196, 97, 5), (2, 16, 46, 4), (2, 157, 43, 5), (3, 23, 9, 4), (3, 217, 44, 5), (4, 85, 44, 5), (4, 133, 69, 4)]
 
 
 @pytest.mark.parametrize("p,nlon,nlat,rows", F32)
