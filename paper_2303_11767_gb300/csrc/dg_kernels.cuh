@@ -1177,18 +1177,24 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // degree 3 220x110 7.3 / 9.4, 260x130 10.2 / 9.6, 360x180 16.5 / 14.4,
     // 1440x720 235 / 202; degree 2 180x90 6.6 / 6.3, 220x110 8.0 / 6.7, 720x360
     // 53.9 / 29.2; degree 1 300x150 4.9 / 5.2, 360x180 7.1 / 5.8, 720x360 18.7 /
-    // 15.2.
+    // 15.2.  At degree 4 the lanes' time jumps where their tiles need a fourth round,
+    // and meshes whose rows are not whole 16-byte blocks take the threads longer
+    // (206x103 14.4 / 16.1 with 455 tiles, 212x107 19.2 / 15.3 with 504), so the line
+    // is at three rounds.
     // It counts the whole mesh's rows, so that a latitude band of a mesh runs
     // the kernel of the whole mesh and gets its bits.
     if constexpr (N >= 2) {
         constexpr long long least = N == 5 ? 21000 : N == 4 ? 32000 : N == 3 ? 18000 : 50000;
-        if ((long long)a.nlon * a.nlat_mesh >= least) {
+        const long long lane_tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((a.nlat_mesh + DG_WARPS - 1) / DG_WARPS);
+        if ((long long)a.nlon * a.nlat_mesh >= least && (N < 5 || lane_tiles > 3 * DG_SMS)) {
             if constexpr (N == 5) {
                 // three tiles run on an SM at a time; where 16 x 8 tiles need a
                 // little more than one round of them, the second round runs nearly
                 // alone, and tiles of 32 x 4, whose last column is cheap, end
                 // sooner (us per stage, 16 x 8 / 32 x 4: 330x165 21.9 / 29.4,
-                // 360x180 33.1 / 30.1, 380x190 34.1 / 30.9, 400x200 35.4 / 41.6)
+                // 360x180 33.1 / 30.1, 380x190 34.1 / 30.9, 400x200 35.4 / 41.6).  After
+                // later rounds the 16 x 8 tiles end sooner all the same (480x240 45.2 /
+                // 48.3, 500x250 57.2 / 60.3, 560x280 67.1 / 73.2, 640x320 85.9 / 90.3)
                 const long long t = ((a.nlon + 15) / 16) * ((a.nlat + 7) / 8);
                 if (t > 3 * DG_SMS && t <= 4 * DG_SMS) return launch_ept_n<5, 32, 4, 3>(a, s);
             }

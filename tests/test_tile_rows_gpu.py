@@ -125,7 +125,7 @@ def tile_rows_f32(nlon, nlat, n):
     return rows
 
 
-F32 = [(0, 162, 37, 8), (0, 206, 93, 8), (0, 299, 149, 5), (4, 196, 97, 8), (1, 7, 15, 4), (1, 141, 67, 8), (1, 196, 97, 5), (2, 16, 46, 4), (2, 157, 43, 5), (3, 23, 9, 4), (3, 217, 44, 5), (4, 85, 44, 5), (4, 133, 69, 4)]
+F32 = [(0, 162, 37, 8), (0, 206, 93, 8), (0, 299, 149, 5), (4, 196, 97, 8), (4, 206, 103, 8), (1, 7, 15, 4), (1, 141, 67, 8), (1, 196, 97, 5), (2, 16, 46, 4), (2, 157, 43, 5), (3, 23, 9, 4), (3, 217, 44, 5), (4, 85, 44, 5), (4, 133, 69, 4)]
 
 
 @pytest.mark.parametrize("p,nlon,nlat,rows", F32)
