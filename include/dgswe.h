@@ -413,6 +413,9 @@ dg_status dg_measure_fp64_peak(int reps, double *gflops);
 
 /* Number of fused stage-kernel launches issued by this handle so far. */
 long long dg_stage_launches(dg_handle h);
+/* Number of CUDA graphs of steps launched by dg_step so far (a call whose step
+ * size comes for the first time launches its stages directly). */
+long long dg_graph_replays(dg_handle h);
 
 /* Message describing the last failing call made by this thread (h may be
  * NULL, e.g. after a failed dg_create); valid until the thread's next call.

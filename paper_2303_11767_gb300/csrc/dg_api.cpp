@@ -62,6 +62,15 @@ struct GraphEntry {
     cudaStream_t stream = nullptr;
 };
 
+constexpr size_t MAX_GRAPHS = 8;   // kept per handle, and recent dg_step calls remembered
+
+struct StepKey {
+    double dt;
+    int rk, prec;
+    cudaStream_t stream;
+    bool operator==(const StepKey &o) const { return dt == o.dt && rk == o.rk && prec == o.prec && stream == o.stream; }
+};
+
 unsigned long long g_basis_uploaded = 0;   // per-device bit: constant tables present
 
 }  // namespace
@@ -107,9 +116,8 @@ struct dg_ctx {
     float *src = nullptr;         // its per-stage modal output
     double *src_part = nullptr;   // and partial sums of the mass in it
     std::vector<GraphEntry> graphs;
-    double last_dt = 0;           // the previous dg_step's key
-    int last_rk = 0, last_prec = 0;
-    cudaStream_t last_stream = nullptr;
+    std::vector<StepKey> recent;  // keys of the latest dg_step calls
+    long long replays = 0;        // graph launches
     double bx = 0, by = 0;       // planar advection velocity
     double plen = 1.0, fcor = 0; // planar domain side and f-plane Coriolis parameter
     int alpha_speed = 0;         // planar: Rusanov alpha = |beta| (1) or |beta . n| (0)
@@ -744,6 +752,8 @@ size_t dg_state_len(dg_handle h) { return h ? h->len : 0; }
 
 long long dg_stage_launches(dg_handle h) { return h ? h->launches : 0; }
 
+long long dg_graph_replays(dg_handle h) { return h ? h->replays : 0; }
+
 const char *dg_last_error(dg_handle) { return g_err.c_str(); }
 
 dg_status dg_set_option(dg_handle h, int key, long long value)
@@ -1014,25 +1024,26 @@ dg_status dg_step(dg_handle h, int n, double dt)
     int K = std::min(h->spg, n);
     if ((K & 1) && K > 1) K -= 1;   // even graphs return u^n to the same base buffer
     int full = n / K, rest = n - full * K;
+    GraphEntry *ge = nullptr;
+    for (auto &g : h->graphs)
+        if (g.steps == K && g.dt == dt && g.order == h->rk && g.prec == h->prec && g.cur_in == h->cur && g.stream == h->stream)
+            ge = &g;
     // A step size that comes for the first time and whose graph this call would
     // replay once (a program that takes its step from the state has a new one
     // each call) is launched directly: capturing and instantiating 16 steps
-    // takes 0.1 ms of host time, the launches hide behind the stages.
-    const bool same = h->last_dt == dt && h->last_rk == h->rk && h->last_prec == h->prec && h->last_stream == h->stream;
-    h->last_dt = dt;
-    h->last_rk = h->rk;
-    h->last_prec = h->prec;
-    h->last_stream = h->stream;
-    if (full == 1 && !same) {
+    // takes 0.1 ms of host time, the launches hide behind the stages.  One that
+    // was among the latest calls is captured, also where several take turns.
+    const StepKey key{dt, h->rk, h->prec, h->stream};
+    const bool seen = std::find(h->recent.begin(), h->recent.end(), key) != h->recent.end();
+    if (!seen) {
+        if (h->recent.size() >= MAX_GRAPHS) h->recent.erase(h->recent.begin());
+        h->recent.push_back(key);
+    }
+    if (!ge && full == 1 && !seen) {
         full = 0;
         rest = n;
     }
     if (full > 0) {
-        GraphEntry *ge = nullptr;
-        for (auto &g : h->graphs)
-            if (g.steps == K && g.dt == dt && g.order == h->rk && g.prec == h->prec && g.cur_in == h->cur &&
-                g.stream == h->stream)
-                ge = &g;
         if (!ge) {
             GraphEntry g;
             g.steps = K;
@@ -1057,7 +1068,7 @@ dg_status dg_step(dg_handle h, int n, double dt)
             cudaGraphDestroy(graph);
             if (ce != cudaSuccess) return fail(DG_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(ce));
             g.cur_out = cur;
-            if (h->graphs.size() >= 8) {
+            if (h->graphs.size() >= MAX_GRAPHS) {
                 cudaGraphExecDestroy(h->graphs.front().exec);
                 h->graphs.erase(h->graphs.begin());
             }
@@ -1069,6 +1080,7 @@ dg_status dg_step(dg_handle h, int n, double dt)
         for (int r = 0; r < full; ++r) {
             CUDA_TRY(cudaGraphLaunch(ge->exec, h->stream));
             h->launches += (long long)K * ns;
+            h->replays++;
             h->cur = ge->cur_out;
         }
     }

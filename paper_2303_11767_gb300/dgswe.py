@@ -54,6 +54,7 @@ SIGNATURES = {
     "dg_get_time": (ctypes.c_int, [_H, _dp]),
     "dg_set_time": (ctypes.c_int, [_H, ctypes.c_double]),
     "dg_stage_launches": (ctypes.c_longlong, [_H]),
+    "dg_graph_replays": (ctypes.c_longlong, [_H]),
     "dg_max_dt_noalloc": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_double,
                                          ctypes.c_double, ctypes.c_double, ctypes.c_void_p, ctypes.c_void_p]),
     "dg_last_error": (ctypes.c_char_p, [_H]),
@@ -371,6 +372,9 @@ class Solver:
 
     def stage_launches(self):
         return int(lib().dg_stage_launches(self._h))
+
+    def graph_replays(self):
+        return int(lib().dg_graph_replays(self._h))
 
     def attach_mlp(self, mlp):
         """Add the network's output as a learned modal source (None detaches)."""
