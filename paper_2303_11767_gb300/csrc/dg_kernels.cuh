@@ -1068,12 +1068,16 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int bx, int by
     if (st && valid) atomicOr(A.status, st);
 }
 
+constexpr int DG_GRID_Y = 65535;   // most blocks in a grid's second dimension
+
 template <typename T, int N, int W, int INC, int FIN>
 __global__ void __launch_bounds__(32 * W) stage_kernel(const StageArgs<T> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_wait();
-    stage_tile<T, N, W, INC, FIN>(A, blockIdx.x, blockIdx.y, smem_raw);
+    const int by = blockIdx.y + DG_GRID_Y * blockIdx.z;
+    if (by * W >= A.nlat) return;   // (the whole block; past the last tile row of a folded grid)
+    stage_tile<T, N, W, INC, FIN>(A, blockIdx.x, by, smem_raw);
     pdl_launch_dependents();
 }
 
@@ -1108,7 +1112,7 @@ int launch_ept_n(const StageArgs<float> &a, cudaStream_t s)
                 return 1;
         attr_set.fetch_or(1ull << dev, std::memory_order_release);   // setting it twice is harmless
     }
-    dim3 grid((a.nlon + TX - 1) / TX, (a.nlat + TY - 1) / TY);
+    const dim3 grid((a.nlon + TX - 1) / TX, (a.nlat + TY - 1) / TY);
     const K k = a.inc ? (a.out_base ? k11 : k10) : (a.out_base ? k01 : k00);
     if (launch_pdl(k, grid, dim3(GE::NT), GE::BYTES, s, a) != cudaSuccess) return 1;
     return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
@@ -1159,7 +1163,9 @@ int launch_stage_w(const StageArgs<T> &a, cudaStream_t s)
                 return 1;
         attr_set.fetch_or(1ull << dev, std::memory_order_release);   // setting it twice is harmless
     }
-    dim3 grid((a.nlon + GE::G - 1) / GE::G, (a.nlat + W - 1) / W);
+    // tile rows beyond a grid's second dimension fold into the third
+    const unsigned rows = (a.nlat + W - 1) / W, nz = (rows + DG_GRID_Y - 1) / DG_GRID_Y;
+    const dim3 grid((a.nlon + GE::G - 1) / GE::G, nz > 1 ? DG_GRID_Y : rows, nz);
     const K k = a.inc ? (a.out_base ? k11 : k10) : (a.out_base ? k01 : k00);
     if (launch_pdl(k, grid, dim3(32 * W), smem, s, a) != cudaSuccess) return 1;
     return cudaPeekAtLastError() == cudaSuccess ? 0 : 1;
@@ -1181,12 +1187,16 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
     // and meshes whose rows are not whole 16-byte blocks take the threads longer
     // (206x103 14.4 / 16.1 with 455 tiles, 212x107 19.2 / 15.3 with 504), so the line
     // is at three rounds.
+    // (Folding its tile rows past 65535 into a third dimension, as launch_stage_w does,
+    // cost 1 to 1.5 %, so meshes of so many rows run the lanes.)
     // It counts the whole mesh's rows, so that a latitude band of a mesh runs
     // the kernel of the whole mesh and gets its bits.
     if constexpr (N >= 2) {
         constexpr long long least = N == 5 ? 21000 : N == 4 ? 32000 : N == 3 ? 18000 : 50000;
         const long long lane_tiles = (long long)((a.nlon + 32 / N - 1) / (32 / N)) * ((a.nlat_mesh + DG_WARPS - 1) / DG_WARPS);
-        if ((long long)a.nlon * a.nlat_mesh >= least && (N < 5 || lane_tiles > 3 * DG_SMS)) {
+        constexpr int TY = N >= 4 ? 8 : 4;
+        if ((long long)a.nlon * a.nlat_mesh >= least && (N < 5 || lane_tiles > 3 * DG_SMS) &&
+            (a.nlat_mesh + TY - 1) / TY <= DG_GRID_Y) {
             if constexpr (N == 5) {
                 // three tiles run on an SM at a time; where 16 x 8 tiles need a
                 // little more than one round of them, the second round runs nearly
@@ -1198,8 +1208,8 @@ int launch_stage_n(const StageArgs<T> &a, cudaStream_t s)
                 const long long t = ((a.nlon + 15) / 16) * ((a.nlat + 7) / 8);
                 if (t > 3 * DG_SMS && t <= 4 * DG_SMS) return launch_ept_n<5, 32, 4, 3>(a, s);
             }
-            if constexpr (N >= 4) return launch_ept_n<N, 16, 8, N == 5 ? 3 : 4>(a, s);
-            else return launch_ept_n<N, 32, 4, N == 3 ? 5 : 6>(a, s);
+            if constexpr (N >= 4) return launch_ept_n<N, 16, TY, N == 5 ? 3 : 4>(a, s);
+            else return launch_ept_n<N, 32, TY, N == 3 ? 5 : 6>(a, s);
         }
     }
 #endif

@@ -142,3 +142,31 @@ def test_short_fp32_tiles(p, nlon, nlat, rows):
         whole = _whole(u, nlon, nlat, p, "fp32", 3, dt, order, torch)[0]
         assert_within(state_err(whole, o.step(u, 3, dt, order)), 1e-5, what)
     assert np.array_equal(_run_bands(u, nlon, nlat, p, "fp32", 2, 3, dt, 4, torch)[0], whole)
+
+
+def _rough(ny, nx, p):
+    rng = np.random.default_rng(3)
+    u = np.zeros((ny, nx, 3, (p + 1) ** 2))
+    u[..., 0, 0] = 2.0 * 5960.0 + rng.normal(size=(ny, nx))
+    u[..., 1:, :] = 1000.0 * rng.normal(size=u[..., 1:, :].shape)
+    return u
+
+
+@pytest.mark.parametrize("p,nlon,nlat,prec", [(1, 2, 262150, "fp32"), (0, 1, 458800, "fp64")])
+def test_more_tile_rows_than_a_grid_dimension(p, nlon, nlat, prec):
+    """Over 65535 tiles of 4 rows (the thread-per-element stage's) and of 7 (FP64).
+    FP64 tolerance: near a pole cos(theta) carries the rounding of theta, 2^-52 nlat / pi of its value."""
+    u = _rough(nlat, nlon, p)
+    o = O.Oracle.sphere(nlon, nlat, p)
+    with dgswe.Solver(nlon, nlat, p, precision=prec) as s:
+        k = s.rhs(u)
+    assert_within(tend_err(k, o.rhs(u), o.rhs_magnitude(u)), 2.0 ** -52 * nlat if prec == "fp64" else 1e-6, f"rhs p={p} {nlon}x{nlat} {prec}")
+
+
+def test_plane_with_more_tile_rows_than_a_grid_dimension():
+    """Tolerance as in test_plane_gpu.py."""
+    u = _rough(524300, 2, 0)
+    with dgswe.Solver.plane_swe(2, 524300, 0, L=1.0e6) as s:
+        k = s.rhs(u)
+    o = O.Oracle.plane_swe(2, 524300, 0, 1.0e6, dgswe.GRAVITY, 1.0e-4)
+    assert_within(tend_err(k, o.rhs(u), o.rhs_magnitude(u)), 1e-12, "plane p=0 2x524300")
