@@ -51,17 +51,15 @@ __device__ __forceinline__ float rcp<float>(float x)
     return y;
 }
 
-template <typename T>
-__device__ __forceinline__ T wave_sqrt(T x);
-template <>
-__device__ __forceinline__ double wave_sqrt<double>(double x) { return sqrt(x); }
-// FP32: x * rsqrt(x) on the SFU; only feeds the Rusanov dissipation speed
-template <>
-__device__ __forceinline__ float wave_sqrt<float>(float x)
+__device__ __forceinline__ double wave_sqrt(double x) { return sqrt(x); }
+// The wave speed |u| + sqrt(gh).  FP32: the root is x * rsqrt(x) on the SFU, its
+// product part of the sum; it only feeds the Rusanov dissipation
+__device__ __forceinline__ double wave_speed(double u, double gh) { return fabs(u) + wave_sqrt(gh); }
+__device__ __forceinline__ float wave_speed(float u, float gh)
 {
     float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return x * y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(gh));
+    return fma(gh, y, fabsf(u));
 }
 
 // Finiteness of many values with one test at the end: chk = fma(x, 0, chk)
@@ -92,10 +90,11 @@ __device__ __forceinline__ void check_depth<double>(double h, unsigned &st)
         st |= (h != h) ? DG_STATUS_NONFINITE : DG_STATUS_NONPHYSICAL;
 }
 
-// Every multiply-add below is an explicit fma: these functions are inlined at
-// several call sites (an edge's flux is evaluated by whichever tile or band
-// owns it), and left to the compiler's contraction the same edge could round
-// differently at two sites.
+// Every multiply-add below is an explicit fma, and every sum that a product
+// enters an explicit addition: these functions are inlined at several call
+// sites (an edge's flux is evaluated by whichever tile or band owns it), and
+// left to the compiler's contraction the same edge could round differently at
+// two sites.
 
 // P = g h' (href + h'/2); FP64 with the constants folded, one operation less
 template <typename T>
@@ -117,7 +116,7 @@ __device__ __forceinline__ void rusanov_out(const T *L, const T *R, const T *fl,
         const T a = aglob > T(0) ? aglob : fmax(al, ar);   // global mode: the stage's largest |u| + c
         const T hc = T(0.5) * c;
 #pragma unroll
-        for (int f = 0; f < 3; ++f) out[f] = hc * fma(-a, R[f] - L[f], fl[f] + fr[f]);
+        for (int f = 0; f < 3; ++f) out[f] = hc * fma(-a, R[f] - L[f], __fadd_rn(fl[f], fr[f]));
     }
 }
 
@@ -134,7 +133,7 @@ __device__ __forceinline__ void lam_flux(const T *q, T href, T g, T *f, T &speed
     f[0] = q[1];
     f[1] = fma(q[1], u, P);
     f[2] = q[2] * u;
-    speed = fabs(u) + wave_sqrt(g * h);
+    speed = wave_speed(u, g * h);
 }
 
 template <typename T>
@@ -147,7 +146,7 @@ __device__ __forceinline__ void th_flux(const T *q, T href, T g, T *f, T &speed,
     f[0] = q[2];
     f[1] = q[1] * v;
     f[2] = fma(q[2], v, P);
-    speed = fabs(v) + wave_sqrt(g * h);
+    speed = wave_speed(v, g * h);
 }
 
 // Rusanov flux through a lambda-face, left state L (west), right state R
