@@ -91,11 +91,18 @@ typedef enum {
     DG_OPT_TILE_ROWS = 7,        /* ensemble only: latitude rows per CTA tile, 4 or 8
                                     (default 8; dg_ensemble_autotune picks it) */
     DG_OPT_BLOCKS_PER_SM = 8,    /* ensemble only: persistent CTAs per SM and degree, 1..8 (default 2) */
-    DG_OPT_WELL_BALANCED = 9     /* 0 (default) / 1: remove from every tendency that of the
+    DG_OPT_WELL_BALANCED = 9,    /* 0 (default) / 1: remove from every tendency that of the
                                     fluid at rest at the reference depth (the mean depth of the
                                     state at dg_set_state), i.e. the quadrature residual of its
                                     constant pressure, so that rest state is exactly steady;
                                     FP64 then also stores h relative to that depth */
+    DG_OPT_BAND_KERNEL = 10      /* latitude bands only: 0 (default): the FP32 stage kernel
+                                    and tile height of the whole mesh, whose state the bands
+                                    then equal bit for bit; 1: those of a mesh of the band's
+                                    own rows, which is faster where the whole mesh's kernel
+                                    is one for many elements and the band has few.  States
+                                    then agree to FP32 rounding; the flux between two bands
+                                    is one value either way.  No effect in FP64 */
 } dg_option;
 
 /* Make CUDA device `device` current for the calling thread in this library

@@ -126,6 +126,7 @@ struct dg_ctx {
     // [j0, j0 + nlat) of a mesh of nlat_g rows; every state array holds, when
     // gs / gn, one ghost row (a neighbour band's row) just before / after them
     int band = 0, j0 = 0, nlat_g = 0, gs = 0, gn = 0;
+    int own_kernel = 0;          // DG_OPT_BAND_KERNEL
     size_t ghost_bytes = 0;    // byte offset of own row 0 in each state allocation
     int band_stage = 0;        // the next stage of the current step
     double band_dt = 0;        // step size of the current step
@@ -203,7 +204,7 @@ StageArgs<T> base_args(dg_ctx *h, const RowTab<T> *rows, double href)
     a.status = h->d_status;
     a.nlon = h->nlon;
     a.nlat = h->nlat;
-    a.nlat_mesh = h->nlat_g;
+    a.nlat_mesh = h->own_kernel && sizeof(T) == sizeof(float) ? h->nlat : h->nlat_g;
     a.halo_s = h->gs;
     a.halo_n = h->gn;
     a.href = (T)href;
@@ -853,6 +854,11 @@ dg_status dg_set_option(dg_handle h, int key, long long value)
     case DG_OPT_STEPS_PER_GRAPH:
         if (value < 1 || value > 1024) return fail(DG_EINVAL, "steps per graph must be 1..1024");
         h->spg = (int)value;
+        return DG_OK;
+    case DG_OPT_BAND_KERNEL:
+        if (!h->band) return fail(DG_EINVAL, "not a band handle");
+        if (value != 0 && value != 1) return fail(DG_EINVAL, "band kernel option must be 0 or 1");
+        h->own_kernel = (int)value;
         return DG_OK;
     default:
         return fail(DG_EINVAL, "unknown option %d", key);

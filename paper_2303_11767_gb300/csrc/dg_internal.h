@@ -97,7 +97,7 @@ struct StageArgs {
     const RowTab<T> *rows;
     unsigned int *status;
     int nlon, nlat;
-    int nlat_mesh;   // rows of the whole mesh (a band's nlat are some of them): the kernel is chosen by it
+    int nlat_mesh;   // rows of the whole mesh (a band's nlat are some of them), or the band's own: the kernel is chosen by it
     // latitude-band sharding: 1 when the row south of row 0 (halo_s) or north
     // of row nlat - 1 (halo_n) is a neighbour band's row, held in the state
     // arrays just before / after the band's own rows, instead of a pole

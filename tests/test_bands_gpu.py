@@ -19,7 +19,7 @@ TOL = {"fp64": 1e-12, "fp32": 1e-5}
 NTHREADS = os.cpu_count() or 1
 
 
-def _run_bands(u0, nlon, nlat, p, prec, nb, nsteps, dt, rk, torch, wb=0):
+def _run_bands(u0, nlon, nlat, p, prec, nb, nsteps, dt, rk, torch, wb=0, own=0):
     stream = torch.cuda.Stream()
     rows = [bands.band_rows(nlat, nb, k) for k in range(nb)]
     bs = [dgswe.Solver.band(nlon, nlat, jb, je, p, R, G, OMEGA, precision=prec, rk_order=rk) for jb, je in rows]
@@ -27,6 +27,7 @@ def _run_bands(u0, nlon, nlat, p, prec, nb, nsteps, dt, rk, torch, wb=0):
     href = bands.reference_depth(None, u0[:, :, 0, 0], 0, 1, torch)
     for b, (jb, je) in zip(bs, rows):
         b.set_option(dgswe.OPT_WELL_BALANCED, wb)
+        b.set_option(dgswe.OPT_BAND_KERNEL, own)
         if prec != "fp64" or wb:
             b.set_reference_depth(href)
         b.set_state(u0[jb:je])

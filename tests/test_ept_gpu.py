@@ -47,6 +47,25 @@ def test_bands_equal_whole_mesh(p, nlon, nlat, nb):
     assert np.array_equal(got, _whole(u, nlon, nlat, p, "fp32", 3, dt, 3, torch)[0])
 
 
+@pytest.mark.parametrize("p,nlon,nlat,nb", [(4, 151, 141, 3), (2, 145, 249, 2), (3, 211, 190, 4), (1, 229, 221, 8)])
+def test_bands_with_their_own_kernel(p, nlon, nlat, nb):
+    """DG_OPT_BAND_KERNEL: bands below the line of a mesh above it (145x249: the bands of 124 and 125 rows
+    lie on both sides of it); other order of sums, so equal to the oracle's states and not to the mesh's bits."""
+    torch = pytest.importorskip("torch")
+    o, u = case(nlon, nlat, p, 11)
+    dt = o.max_dt(u, 0.1)
+    with dgswe.Solver.band(nlon, nlat, 0, 9, p, precision="fp32") as b, dgswe.Solver(9, 5, 1) as s:
+        for handle, value in ((b, 2), (b, -1), (s, 1)):
+            with pytest.raises(dgswe.DGError) as e:
+                handle.set_option(dgswe.OPT_BAND_KERNEL, value)
+            assert e.value.status == dgswe.DG_EINVAL
+    got, mass, _ = _run_bands(u, nlon, nlat, p, "fp32", nb, 3, dt, 3, torch, own=1)
+    want, whole_mass, _ = _whole(u, nlon, nlat, p, "fp32", 3, dt, 3, torch)
+    assert not np.array_equal(got, want)   # the other kernel ran
+    assert_within(state_err(got, o.step(u, 3, dt, 3)), 1e-5, f"own kernel p={p} {nlon}x{nlat}")
+    assert abs(mass / whole_mass - 1) < 1e-9   # FP32 increments of the mean depth
+
+
 @pytest.mark.parametrize("j,i", [(0, 0), (140, 150), (57, 64)])
 @pytest.mark.parametrize("value,status", [(np.nan, dgswe.DG_ENONFINITE), (-3.0e4, dgswe.DG_ENONPHYSICAL)])
 def test_bad_state_is_reported(j, i, value, status):
