@@ -596,9 +596,10 @@ namespace {
 // the total from mode (0, 0) of h, spread over the area.
 //
 // The weights (51 KB) are read once per block before the wait for the previous
-// stage, so S is the smallest size that gives every SM at most one block.  At
-// 72x36, per stage: one thread per hidden unit reading its own weight row 46 us
-// and a single-block mass sum 13 us; now 15 us with the stage.
+// stage, so S is the smallest of 8, 12, 20 and 32 that gives every SM at most one
+// block, and 32 for meshes that need several rounds.  At 72x36, per stage: one thread per
+// hidden unit reading its own weight row 46 us and a single-block mass sum 13 us; now
+// 15 us with the stage.
 constexpr int SRC_KS = 4;
 
 // One hidden layer of the source block: A -> gelu(A W + b) (K inputs), the

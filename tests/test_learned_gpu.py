@@ -137,6 +137,66 @@ def test_learned_source_matches_reference_and_keeps_mass():
         assert abs(s.total_mass() / m0 - 1) < 1e-8
 
 
+# the source kernel's four block sizes (8, 12, 20, 32 elements), each with an odd number of columns and a
+# ragged last block, and meshes whose stage runs one thread per element
+SIZES = [(31, 17), (57, 29), (73, 36), (181, 91), (317, 159), (229, 221)]
+
+
+@pytest.mark.parametrize("nlon,nlat", SIZES)
+def test_source_at_every_block_size(nlon, nlat):
+    """The source in the tendency, its mass, and two SSP-RK3 steps against the FP64 network and oracle.
+    Tolerances: network outputs 1e-5 of the largest (as in test_mlp_gpu.py; 1e-4 after the steps, whose later
+    inputs carry the FP32 state's rounding), FP32 tendencies 1e-6 of their magnitude bound."""
+    o = O.Oracle.sphere(nlon, nlat, 1, R, G, OMEGA)
+    u = o.project_tensor(synth.SmoothField(21).fields_grid)
+    X = learned.gather_inputs(u)
+    std = (X.std(0) + 1e-6 * np.abs(X).max()).astype(np.float32)
+    mlp = dgswe.MLP(60, 128, 12, seed=2)
+    dt = o.max_dt(u, 0.1)
+    ys = (0.02 * std[:12] / dt).astype(np.float32)   # a step changes the inputs by a part of their spread
+    mlp.set_normalization(X.mean(0), std, np.zeros(12, np.float32), ys)
+    p = mlp.get_params()
+    p += np.random.default_rng(5).normal(scale=0.01, size=p.shape).astype(np.float32)   # biases too
+    mlp.set_params(p)
+    nrm = (X.mean(0).astype(np.float32).astype(np.float64), std.astype(np.float64), np.zeros(12), ys.astype(np.float64))
+    c0 = np.array([[o.mass_matrix(j)[0, 0], o.mass_matrix(j)[0, 2]] for j in range(nlat)])
+
+    def mass(v):
+        return (c0[:, None, 0] * v[..., 0, 0] + c0[:, None, 1] * v[..., 0, 2]).sum()
+
+    def source(v):
+        y, _ = M.forward(p.astype(np.float64), learned.gather_inputs(v), nrm, 60, 128, 12)
+        src = (y * nrm[3]).reshape(nlat, nlon, 3, 4)
+        src[..., 0, 0] -= mass(src) / (c0[:, 0].sum() * nlon)
+        return src
+
+    def step(v, dt, f):   # SSP-RK3
+        k1 = f(v)
+        k2 = f(v + dt * k1)
+        return v + dt / 6 * (k1 + k2 + 4 * f(v + 0.25 * dt * (k1 + k2)))
+
+    out = []
+    with dgswe.Solver(nlon, nlat, 1, R, G, OMEGA, precision="fp32") as s:
+        for net in (None, mlp):
+            s.attach_mlp(net)
+            k = s.rhs(u)
+            s.set_state(u)
+            s.step(2, dt)
+            out.append((k, s.get_state()))
+        s.attach_mlp(None)
+    src, S = source(u), o.rhs_magnitude(u)
+    d = out[1][0] - out[0][0]
+    for f in range(3):
+        assert np.abs(d - src)[..., f, :].max() < 1e-5 * np.abs(src[..., f, :]).max() + 2e-6 * S[..., f, :].max()
+    added = sum(np.abs(c0[:, None, i] * src[..., 0, 2 * i]).sum() for i in range(2))
+    assert abs(mass(d)) < 1e-5 * added + 2e-6 * (c0[:, 0] * S[..., 0, 0].sum(1)).sum()
+    want = step(step(u, dt, lambda v: o.rhs(v) + source(v)), dt, lambda v: o.rhs(v) + source(v))
+    plain = step(step(u, dt, o.rhs), dt, o.rhs)
+    d, ref = out[1][1] - out[0][1], want - plain
+    for f in range(3):
+        assert np.abs(d - ref)[..., f, :].max() < 1e-4 * np.abs(2 * dt * src[..., f, :]).max() + 4e-6 * dt * S[..., f, :].max()
+
+
 def test_row_normalised_source_matches_reference():
     o, u = _coarse_state()
     mlp = dgswe.MLP(60, 128, 12, seed=3)
