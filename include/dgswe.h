@@ -173,7 +173,8 @@ dg_status dg_rhs(dg_handle h, const double *modal_in, double *tend_out, size_t l
 
 /* Advance the resident state by n >= 0 steps of size dt > 0 with the SSP
  * Runge-Kutta scheme of order DG_OPT_RK_ORDER (Table "Butcher"), replaying a
- * captured CUDA graph of fused stage kernels.  Adds n*dt to the simulated
+ * captured CUDA graph of fused stage kernels (or launching them directly where
+ * the step size is not among the latest calls').  Adds n*dt to the simulated
  * time.  With DG_OPT_CHECK_FINITE, synchronises and reports DG_ENONFINITE or
  * DG_ENONPHYSICAL if any stage met a non-finite value or h <= 0. */
 dg_status dg_step(dg_handle h, int n, double dt);
